@@ -1262,7 +1262,7 @@ int fg_rotate(fg_ctx *ctx, const fg_keys *keys, const uint64_t *ct, int level, i
     u64 *digits = (u64 *)ctx->buf("rot_digits",
                                   (size_t)ctx->n_digits(level) * ctx->ext(level) * N * 8);
     kern::modup(ctx, lane, nl, 1, level, digits);
-    kern::rotate_mac(ctx, key, lane, nl, 1, level, digits, {{res, nullptr}}, nl);
+    kern::rotate(ctx, key, lane, nl, 1, level, digits, res, nl);
     kern::LimbSet rs{res, nl, nl, 2, pid};
     kern::ntt_inv(ctx, rs, rs);
     stage_out(ctx, out, res, (size_t)2 * nl * N);

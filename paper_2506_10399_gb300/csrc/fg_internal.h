@@ -101,9 +101,9 @@ struct Tune {
     int ks_cols = 1;       // key switch: launches the columns are split over (1 or 2)
     int modup_fused = 1;   // N = 2^16 ModUp: 1 = conversion fused into the digits' first NTT pass
     int moddown_fused = 0; // N = 2^16 ModDown + rescale: 1 = conversion fused into the first NTT pass
-    int gmac_groups = 7;   // group MAC: outputs from which a CTA runs three thread groups
-    int gmac_regs = 1;     // group MAC: 1 = registers for 3 CTAs of 384 threads per SM, 0 = for 2
-    int kara = 1;          // group MAC, split products below 2^46: 1 = three products
+    int gmac_groups = 7;   // group MAC, tiled form: outputs from which a CTA runs three thread groups
+    int gmac_regs = 1;     // group MAC, tiled form: 1 = registers for 3 CTAs of 384 threads per SM, 0 = for 2
+    int kara = 1;          // group MAC, tiled form, split products below 2^46: 1 = three products
                            // (Karatsuba), 0 = four
     bool operator==(const Tune &o) const
     {
@@ -235,7 +235,8 @@ struct MaskC {
     int level;
     std::vector<int32_t> slots;   // sorted
     std::vector<double> values;
-    u64 *d = nullptr;             // [level+1][N] NTT domain, Montgomery form
+    bool kept = false;            // mask of a group's kept values: stored times P, zero mod the special primes
+    u64 *d = nullptr;             // [E][N] NTT domain, Montgomery form, split halves (split_word)
 };
 
 struct fg_plan {
@@ -278,7 +279,10 @@ void ntt_fwd(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst);
 void ntt_inv(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst);
 
 // contiguous [count][N] limbs, limb c modulo prime pidx[c % pidx.size()]
-void to_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx);
+// split: words left as split halves (split_word), the form of plan masks;
+// times_p: limbs of Q times P, the special primes' limbs zero
+void to_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx, bool split = false,
+             bool times_p = false);
 void from_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx);
 void pointwise(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count,
                const std::vector<int> &pidx);
@@ -310,23 +314,23 @@ void rescale_ntt(fg_ctx *ctx, u64 *ct, int ls, int npoly, int level);
 // ModUp of the c1 parts of ncol ciphertexts (NTT domain, limb stride ls) at
 // `level`: digits [ncol][beta][E][N], NTT domain, own-digit limbs not written
 void modup(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level, u64 *digits);
+// out = Rot(lane, k) from the hoisted digits
+void rotate(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, int level, const u64 *digits, u64 *out,
+            int out_ls);
 struct Dest {
     u64 *out;          // accumulator ciphertexts (limb stride out_ls)
-    const u64 *mask;   // [level+1][N] NTT domain, Montgomery form; null = store R
+    const u64 *mask;   // [level+1][N] NTT domain, Montgomery form, split halves
 };
-// R = Rot(lane, k) from the hoisted digits; every destination gets mask (x) R
-void rotate_mac(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, int level,
-                const u64 *digits, const std::vector<Dest> &dests, int out_ls);
-// every destination gets mask (x) lane
 struct GroupSource {
     const u64 *u;      // rotation: key-switch output [ncol][2][E][N]; kept lane: nullptr
     const u64 *lane;   // the source lane
     uint32_t galois;
     int t0, t1;        // its terms (indices into the term list)
 };
-// one SpIntra-CA group's outputs in the extended basis (see k_group_mac);
-// a launch takes at most kGmacSrc sources and kGmacTerms terms
+// one SpIntra-CA group's outputs in the extended basis (see gmac.cu); a
+// launch takes at most kGmacSrc sources, kGmacOut outputs and kGmacTerms terms
 constexpr int kGmacSrc = 36;
+constexpr int kGmacOut = 64;
 constexpr int kGmacTerms = 300;
 void group_mac(fg_ctx *ctx, const std::vector<GroupSource> &srcs, const std::vector<Dest> &terms,
                const std::vector<int> &term_dest, const std::vector<u64 *> &outs, bool accumulate,
@@ -340,6 +344,7 @@ void ks_multi(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::v
 void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls);
 // residues mod the special primes from limb 0 (centred): out [np][N]
 void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out);
+// every destination gets mask (x) lane
 void stay_mac(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level,
               const std::vector<Dest> &dests, int out_ls);
 }  // namespace kern

@@ -675,15 +675,22 @@ __device__ __forceinline__ const u64 *limb_ptr(const u64 *base, int stride, int 
     return base + ((size_t)(limb / per_row) * stride + (limb % per_row)) * N;
 }
 
-__global__ void k_to_mont(const Batch bt, const PrimeC *__restrict__ primes, int N)
+// split: the words are left as split halves (split_word), the form in which
+// the group MAC and the masked products take plan masks; pmodq: a mask of
+// kept values, its limbs of Q (prime index below nq) times P, the others 0
+__global__ void k_to_mont(const Batch bt, const PrimeC *__restrict__ primes, int N, int split,
+                          const u64 *__restrict__ pmodq, int nq)
 {
     const int limb = blockIdx.y;
     const int pi = bt.pidx[limb % bt.per_row];
     if (pi < 0) return;
     const PrimeC P = primes[pi];
     u64 *d = const_cast<u64 *>(limb_ptr(bt.dst, bt.dst_stride, bt.per_row, limb, N));
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N; x += gridDim.x * blockDim.x)
-        d[x] = mont_mul(d[x], P.r2, P);
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N; x += gridDim.x * blockDim.x) {
+        u64 m = mont_mul(d[x], P.r2, P);
+        if (pmodq) m = pi < nq ? shoup_mul(m, pmodq[2 * pi], pmodq[2 * pi + 1], P.q) : 0;
+        d[x] = split ? split_word(m, P.q) : m;
+    }
 }
 
 __global__ void k_from_mont(const Batch bt, const PrimeC *__restrict__ primes, int N)
@@ -1171,38 +1178,22 @@ k_ks_ip(const KsSet ks, int KL, const u64 *__restrict__ lane, int ls,
 }
 
 // ------------------------------------------------------------------------
-// ModDown finish + masked accumulation (the SpIntra-CA products):
-//   R_p = (u_p - conv_p) * P^-1  (+ phi_g(c0) for p = 0)
-//   out_d += mask_d (x) R         (mask in Montgomery form; null mask: out_d = R)
+// ModDown finish of one rotation:
+//   out_p = (u_p - conv_p) * P^-1  (+ phi_g(c0) for p = 0)
 // ------------------------------------------------------------------------
-constexpr int kMaxDest = 8;
-struct DestList {
-    int n;
-    int out_ls;
-    u64 *out[kMaxDest];
-    const u64 *mask[kMaxDest];
-};
-
 __global__ void __launch_bounds__(256)
-k_moddown_finish_mac(const u64 *__restrict__ u, int E, const u64 *__restrict__ conv,
-                     const u64 *__restrict__ lane, int ls, int ncol, int level, uint32_t g,
-                     int log_n, const u64 *__restrict__ pinv, const DestList dl,
-                     const PrimeC *__restrict__ primes)
+k_moddown_finish(const u64 *__restrict__ u, int E, const u64 *__restrict__ conv, const u64 *__restrict__ lane, int ls,
+                 int ncol, int level, uint32_t g, int log_n, const u64 *__restrict__ pinv, u64 *out, int out_ls,
+                 const PrimeC *__restrict__ primes)
 {
     const int N = 1 << log_n;
     const int i = blockIdx.y;
     const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x >= N) return;
-    const PrimeC P = primes[i];
-    const u64 q = P.q, pv = pinv[2 * i], pvs = pinv[2 * i + 1];
+    const u64 q = primes[i].q, pv = pinv[2 * i], pvs = pinv[2 * i + 1];
     const int sx = auto_src(x, g, log_n);
     const bool swap = sx & 1;
     const int nl = level + 1;
-    ulonglong2 m[kMaxDest];
-#pragma unroll
-    for (int d = 0; d < kMaxDest; d++)
-        if (d < dl.n && dl.mask[d])
-            m[d] = *reinterpret_cast<const ulonglong2 *>(dl.mask[d] + (size_t)i * N + x);
     for (int f = 0; f < ncol; f++) {
 #pragma unroll
         for (int p = 0; p < 2; p++) {
@@ -1216,23 +1207,18 @@ k_moddown_finish_mac(const u64 *__restrict__ u, int E, const u64 *__restrict__ c
                 r0 = add_mod(r0, c0.x, q);
                 r1 = add_mod(r1, c0.y, q);
             }
-#pragma unroll
-            for (int d = 0; d < kMaxDest; d++) {
-                if (d < dl.n) {
-                    ulonglong2 *o = reinterpret_cast<ulonglong2 *>(dl.out[d] + ((size_t)poly * dl.out_ls + i) * N + x);
-                    if (dl.mask[d]) {
-                        ulonglong2 ov = *o;
-                        ov.x = add_mod(ov.x, mont_mul(r0, m[d].x, P), q);
-                        ov.y = add_mod(ov.y, mont_mul(r1, m[d].y, P), q);
-                        *o = ov;
-                    } else {
-                        *o = make_ulonglong2(r0, r1);
-                    }
-                }
-            }
+            *reinterpret_cast<ulonglong2 *>(out + ((size_t)poly * out_ls + i) * N + x) = make_ulonglong2(r0, r1);
         }
     }
 }
+
+constexpr int kMaxDest = 8;
+struct DestList {
+    int n;
+    int out_ls;
+    u64 *out[kMaxDest];
+    const u64 *mask[kMaxDest];
+};
 
 // out_d += mask_d (x) lane (the kept values of a lane, rotation 0)
 __global__ void __launch_bounds__(256)
@@ -1246,7 +1232,10 @@ k_stay_mac(const u64 *__restrict__ lane, int ls, int ncol, int level, const Dest
     ulonglong2 m[kMaxDest];
 #pragma unroll
     for (int d = 0; d < kMaxDest; d++)
-        if (d < dl.n) m[d] = *reinterpret_cast<const ulonglong2 *>(dl.mask[d] + (size_t)i * N + x);
+        if (d < dl.n) {
+            m[d] = *reinterpret_cast<const ulonglong2 *>(dl.mask[d] + (size_t)i * N + x);
+            m[d] = make_ulonglong2(join_word(m[d].x, P.q), join_word(m[d].y, P.q));
+        }
     for (int f = 0; f < ncol; f++) {
 #pragma unroll
         for (int p = 0; p < 2; p++) {
@@ -1263,211 +1252,6 @@ k_stay_mac(const u64 *__restrict__ lane, int ls, int ncol, int level, const Dest
                 }
             }
         }
-    }
-}
-
-// ------------------------------------------------------------------------
-// One SpIntra-CA group, all outputs at once (double hoisting): for each
-// output d,  ext_d = sum over its rotated sources r of mask (x) (u_r +
-// P phi_r(c0)) + sum over its kept sources of mask (x) P lane, in the
-// extended basis q_0..q_l, p_0..p_{K-1} (the P terms vanish mod p_k).
-// ModDown(ext_d) is then exactly the sum of mask (x) Rot and mask (x) lane,
-// since ModDown(A + P B) = ModDown(A) + B.
-// ------------------------------------------------------------------------
-
-// Partial sums are products v * m~ (m~ = mask R mod q, its Montgomery form)
-// added without reduction; one Montgomery reduction of the total gives
-// sum v * m mod q.  That needs total < q 2^64: every product is below
-// q^2 < 2^120, so up to 255 terms per output and launch are safe after
-// folding the high word mod q (a launch takes at most kGmacSrc sources, and
-// each source feeds an output at most once).
-//
-// For primes below 2^46 both factors are split into 23-bit halves,
-// v = v0 + v1 2^23, and the three partial sums  A0 = sum v0 m0,
-// A1 = sum (v0 m1 + v1 m0), A2 = sum v1 m1  are kept in 64-bit words
-// (below 2^55 for 255 terms): four 32 x 32 -> 64-bit multiply-adds per
-// product instead of a 64 x 64 -> 128-bit one.  The halves are stored as
-// v0 | v1 << 32, so each factor is a register pair read without shifts.
-// Other primes (q_0 and the special primes, up to 60 bits) are split into
-// 30-bit halves and folded into a 128-bit sum every 8 terms.
-//
-// Tiling.  A tile is PPC polynomials (column, part) times PPN neighbouring
-// slot pairs of one limb, thread = one polynomial at one slot pair (PPC =
-// min(npoly, 16), PPN = min(128 / PPC, 16): for 32 polynomials two tiles of
-// 16 x 8, 128-byte runs per polynomial).  A CTA holds one tile and G thread
-// groups that share its staged words: every group copies and splits a share
-// of the sources and masks, then computes its own contiguous slice of the
-// outputs (balanced by term count on the host).  With seven or more outputs
-// G = 3: the CTA gets three times the warps for the same shared memory
-// (measured on a 66-source, 12-output group: 9% faster than one group);
-// with fewer, the per-thread setup of extra groups costs more than it
-// hides (6 outputs: one group 20% faster than three), so G = 1.  Phase 1
-// copies the sources (the key-switch output, which already holds u +
-// P phi(c0), or the kept lane) and the tile's mask words into shared memory
-// with asynchronous copies, all in flight at once; phase 2 turns kept lanes
-// into P lane and splits words in place; phase 3 walks the group's
-// outputs, each a register sum over its terms.
-constexpr int kGmacTile = 128;    // threads per group: PPC x PPN (idle ones when npoly < 8)
-constexpr int kGmacGroups = 3;    // most output groups per CTA
-constexpr int kGmacThreads = kGmacTile * kGmacGroups;
-constexpr int kGmacOut = 64;      // outputs per launch
-
-// the launch's program, passed by value (kernel parameters sit in the
-// constant bank: uniform reads need no global loads)
-struct GProg {
-    int nsrc, nterm, X, accumulate;
-    int ppc, ppn;                       // tile: polynomials x slot pairs
-    int groups;                         // thread groups (blockDim = groups x kGmacTile)
-    int gfirst[kGmacGroups + 1];        // first output of each thread group
-    const u64 *su[kern::kGmacSrc];      // rotation: key-switch output; kept lane: nullptr
-    const u64 *slane[kern::kGmacSrc];   // kept lane
-    u32 tvoff[kern::kGmacTerms];        // terms sorted by output: byte offset of the source's row in vsm
-    const u64 *tmask[kern::kGmacTerms];
-    int dfirst[kGmacOut + 1];
-    u64 *outs[kGmacOut];
-};
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
-// 16-byte shared-memory load by 32-bit shared address (volatile: it must
-// stay after the barrier that publishes the staged words)
-__device__ __forceinline__ ulonglong2 lds128(u32 addr)
-{
-    ulonglong2 v;
-    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(addr));
-    return v;
-}
-
-// MINB: CTAs of kGmacThreads threads per SM the registers are budgeted for
-// (2: up to 85 registers a thread; 3: up to 56, more warps resident).
-// KARA: the 23-bit split products in Karatsuba's form (mac_kara: three
-// products instead of four; the same sums).
-template <int MINB, bool KARA>
-__global__ void __launch_bounds__(kGmacThreads, MINB)
-k_group_mac(const GProg pg, int ncol, int level, int E, int ls, int log_n,
-            const u64 *__restrict__ pmodq, const PrimeC *__restrict__ primes, int nq)
-{
-    extern __shared__ __align__(16) unsigned char gsm[];
-    const int npoly = 2 * ncol, PPC = pg.ppc, PPN = pg.ppn;
-    const int npg = (npoly + PPC - 1) / PPC;
-    const int nsrc = pg.nsrc, nterm = pg.nterm;
-    ulonglong2 *vsm = reinterpret_cast<ulonglong2 *>(gsm);                  // [nsrc][kGmacTile]
-    ulonglong2 *msm = vsm + (size_t)nsrc * kGmacTile;                       // [nterm][PPN]
-    const int N = 1 << log_n;
-    const int grp = threadIdx.x / kGmacTile, lt = threadIdx.x % kGmacTile;
-    const int pl = lt / PPN, pp = lt - pl * PPN;
-    const int pgi = blockIdx.x % npg, blk = blockIdx.x / npg;
-    const int poly = pgi * PPC + pl;
-    const int x = 2 * (blk * PPN + pp);
-    const bool xin = pl < PPC && x < N;          // a slot pair of the tile
-    const bool act = xin && poly < npoly;        // ... of an existing polynomial
-    const int i = blockIdx.y;
-    const bool isq = i <= level;
-    const PrimeC P = primes[isq ? i : nq + (i - level - 1)];
-    const u64 q = P.q;
-    const bool split = q < (1ull << 46);
-    const size_t ext_off = ((size_t)poly * E + i) * N + x;
-    const int G = pg.groups;
-    // 1. asynchronous copies: the masks of terms grp PPC + pl (step G PPC)
-    // at this slot pair, the sources grp, grp + G, ... of this thread's slot
-    if (xin)
-        for (int t = grp * PPC + pl; t < nterm; t += G * PPC)
-            cp_async16(msm + t * PPN + pp, pg.tmask[t] + (size_t)i * N + x);
-    if (act) {
-        for (int s = grp; s < nsrc; s += G) {
-            ulonglong2 *dst = vsm + (size_t)s * kGmacTile + lt;
-            if (pg.su[s]) cp_async16(dst, pg.su[s] + ext_off);
-            else if (isq) cp_async16(dst, pg.slane[s] + ((size_t)poly * ls + i) * N + x);
-            else *dst = make_ulonglong2(0, 0);   // P lane vanishes mod the special primes
-        }
-    }
-    cp_async_wait_all();
-    // 2. in place, each thread on the words it copied: kept lanes times P,
-    // every word split into halves (23 bits below 2^46, else 30 bits)
-    if (xin)
-        for (int t = grp * PPC + pl; t < nterm; t += G * PPC) {
-            const ulonglong2 m = msm[t * PPN + pp];
-            msm[t * PPN + pp] = split ? make_ulonglong2(split23(m.x), split23(m.y))
-                                      : make_ulonglong2(split30(m.x), split30(m.y));
-        }
-    if (act) {
-        const u64 pw = isq ? pmodq[2 * i] : 0, pws = isq ? pmodq[2 * i + 1] : 0;
-        for (int s = grp; s < nsrc; s += G) {
-            const bool kept = isq && !pg.su[s];
-            ulonglong2 *dst = vsm + (size_t)s * kGmacTile + lt;
-            ulonglong2 v = *dst;
-            if (kept) {
-                v.x = shoup_mul(v.x, pw, pws, q);
-                v.y = shoup_mul(v.y, pw, pws, q);
-            }
-            *dst = split ? make_ulonglong2(split23(v.x), split23(v.y))
-                         : make_ulonglong2(split30(v.x), split30(v.y));
-        }
-    }
-    __syncthreads();
-    if (!act) return;
-    // 3. this group's outputs.  Shared-memory reads by 32-bit address: the
-    // source row of a term is a constant offset from this thread's slot, the
-    // mask row steps by PPN words per term.
-    const int d0 = pg.gfirst[grp], d1 = pg.gfirst[grp + 1];
-    const u32 vbase = (u32)__cvta_generic_to_shared(vsm + lt);
-    const u32 mstep = (u32)PPN * 16;
-    u32 maddr = (u32)__cvta_generic_to_shared(msm + pp) + (u32)pg.dfirst[d0] * mstep;
-    for (int d = d0; d < d1; d++) {
-        ulonglong2 *o = reinterpret_cast<ulonglong2 *>(pg.outs[d] + ext_off);
-        const ulonglong2 b = pg.accumulate ? *o : make_ulonglong2(0, 0);
-        const int t0 = pg.dfirst[d], t1 = pg.dfirst[d + 1];
-        ulonglong2 r;
-        if (split) {
-            u64 a0 = 0, a1 = 0, a2 = 0, c0 = 0, c1 = 0, c2 = 0;
-            if (KARA) {
-                for (int t = t0; t < t1; t++, maddr += mstep) {
-                    const ulonglong2 v = lds128(vbase + pg.tvoff[t]);
-                    const ulonglong2 m = lds128(maddr);
-                    mac_kara(a0, a1, a2, v.x, m.x);
-                    mac_kara(c0, c1, c2, v.y, m.y);
-                }
-                r = make_ulonglong2(fold_kara(a0, a1, a2, P), fold_kara(c0, c1, c2, P));
-            } else {
-                for (int t = t0; t < t1; t++, maddr += mstep) {
-                    const ulonglong2 v = lds128(vbase + pg.tvoff[t]);
-                    const ulonglong2 m = lds128(maddr);
-                    mac_split(a0, a1, a2, v.x, m.x);
-                    mac_split(c0, c1, c2, v.y, m.y);
-                }
-                r = make_ulonglong2(fold_split(a0, a1, a2, P), fold_split(c0, c1, c2, P));
-            }
-        } else {
-            // 30-bit halves: partial sums folded into 128 bits every 8 terms
-            u64 lo0 = 0, hi0 = 0, lo1 = 0, hi1 = 0;
-            for (int t = t0; t < t1;) {
-                const int te = min(t + 8, t1);
-                u64 a0 = 0, a1 = 0, a2 = 0, c0 = 0, c1 = 0, c2 = 0;
-                for (; t < te; t++, maddr += mstep) {
-                    const ulonglong2 v = lds128(vbase + pg.tvoff[t]);
-                    const ulonglong2 m = lds128(maddr);
-                    mac_split(a0, a1, a2, v.x, m.x);
-                    mac_split(c0, c1, c2, v.y, m.y);
-                }
-                fold30(hi0, lo0, a0, a1, a2);
-                fold30(hi1, lo1, c0, c1, c2);
-            }
-            r = make_ulonglong2(redc(reduce_word(hi0, P), lo0, P), redc(reduce_word(hi1, P), lo1, P));
-        }
-        if (pg.accumulate) {
-            r.x = add_mod(r.x, b.x, q);
-            r.y = add_mod(r.y, b.y, q);
-        }
-        *o = r;
     }
 }
 
@@ -1774,12 +1558,13 @@ static Batch contiguous(u64 *p, int count, const std::vector<int> &pidx)
     return make_batch(p, per, p, per, per, count / per, pidx);
 }
 
-void to_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx)
+void to_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx, bool split, bool times_p)
 {
     if (!count) return;
     KTimer kt(ctx, "to_mont", 0);
     k_to_mont<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(contiguous(data, count, pidx),
-                                                               ctx->d_primes, ctx->n);
+                                                               ctx->d_primes, ctx->n, split ? 1 : 0,
+                                                               times_p ? ctx->d_pmodq : nullptr, ctx->nq);
     check_launch("to_mont");
 }
 
@@ -2048,8 +1833,8 @@ static void ks_launch(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, cons
     check_launch("ks_ip");
 }
 
-void rotate_mac(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, int level,
-                const u64 *digits, const std::vector<Dest> &dests, int out_ls)
+void rotate(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, int level, const u64 *digits, u64 *out,
+            int out_ls)
 {
     const int N = ctx->n, nl = level + 1, E = ctx->ext(level), beta = ctx->n_digits(level);
     FG_CHECK(beta <= kMaxBeta, FG_EINVAL, "too many key-switching digits");
@@ -2075,26 +1860,11 @@ void rotate_mac(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int nco
     for (int i = 0; i < nl; i++) pq[i] = i;
     LimbSet cs{conv, nl, nl, 2 * ncol, pq};
     ntt_fwd(ctx, cs, cs);
-    for (size_t d0 = 0; d0 < dests.size() || d0 == 0; d0 += kMaxDest) {
-        DestList dl;
-        dl.n = (int)std::min<size_t>(kMaxDest, dests.size() - d0);
-        dl.out_ls = out_ls;
-        for (int d = 0; d < dl.n; d++) {
-            dl.out[d] = dests[d0 + d].out;
-            dl.mask[d] = dests[d0 + d].mask;
-        }
-        dim3 g3((N / 2 + 255) / 256, nl);
-        int masked = 0;
-        for (int d = 0; d < dl.n; d++) masked += dl.mask[d] != nullptr;
-        KTimer kt(ctx, "moddown_mac",
-                  ((double)5 * ncol * nl + (double)masked * nl +
-                   (double)masked * ncol * 2 * nl * 2 + (double)(dl.n - masked) * ncol * 2 * nl) * N * 8);
-        k_moddown_finish_mac<<<g3, 256, 0, ctx->stream>>>(u, E, conv, lane, ls, ncol, level,
-                                                          key.galois, ctx->log_n,
-                                                          ctx->pinv_tab(level), dl, ctx->d_primes);
-        check_launch("moddown_finish_mac");
-        if (dests.empty()) break;
-    }
+    dim3 g3((N / 2 + 255) / 256, nl);
+    KTimer kt(ctx, "moddown_mac", (double)7 * ncol * nl * N * 8);
+    k_moddown_finish<<<g3, 256, 0, ctx->stream>>>(u, E, conv, lane, ls, ncol, level, key.galois, ctx->log_n,
+                                                  ctx->pinv_tab(level), out, out_ls, ctx->d_primes);
+    check_launch("moddown_finish");
 }
 
 void stay_mac(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level,
@@ -2126,74 +1896,6 @@ void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out)
                                                                       ctx->np, ctx->nq,
                                                                       ctx->d_primes, ctx->n);
     check_launch("lift_special");
-}
-
-void group_mac(fg_ctx *ctx, const std::vector<GroupSource> &srcs, const std::vector<Dest> &terms_in,
-               const std::vector<int> &term_dest, const std::vector<u64 *> &outs, bool accumulate,
-               int ncol, int level, int ls)
-{
-    const int N = ctx->n, E = ctx->ext(level), X = (int)outs.size();
-    if (srcs.empty() || X == 0) return;
-    FG_CHECK((int)srcs.size() <= kGmacSrc && (int)terms_in.size() <= kGmacTerms && X <= kGmacOut,
-             FG_EINVAL, "group_mac: launch larger than its program limits");
-    GProg pg;
-    memset(&pg, 0, sizeof(pg));
-    pg.nsrc = (int)srcs.size();
-    pg.nterm = (int)terms_in.size();
-    pg.X = X;
-    pg.accumulate = accumulate ? 1 : 0;
-    std::vector<int> src_of(terms_in.size());
-    for (size_t s = 0; s < srcs.size(); s++) {
-        pg.su[s] = srcs[s].u;
-        pg.slane[s] = srcs[s].lane;
-        for (int t = srcs[s].t0; t < srcs[s].t1; t++) src_of[t] = (int)s;
-    }
-    int n = 0;
-    for (int d = 0; d < X; d++) {   // terms sorted by output
-        pg.dfirst[d] = n;
-        pg.outs[d] = outs[d];
-        for (size_t t = 0; t < terms_in.size(); t++)
-            if (term_dest[t] == d) {
-                pg.tvoff[n] = (u32)src_of[t] * kGmacTile * 16;
-                pg.tmask[n] = terms_in[t].mask;
-                n++;
-            }
-    }
-    pg.dfirst[X] = n;
-    // thread groups and their output slices, cut where the running term
-    // count passes k / G of the total
-    const int G = X >= ctx->tune.gmac_groups ? kGmacGroups : 1;
-    pg.groups = G;
-    pg.gfirst[0] = 0;
-    int k = 1;
-    for (int d = 0; d < X && k < G; d++)
-        while (k < G && (int64_t)pg.dfirst[d + 1] * G >= (int64_t)k * n) pg.gfirst[k++] = d + 1;
-    for (; k <= kGmacGroups; k++) pg.gfirst[k] = X;
-    const int npoly = 2 * ncol;
-    pg.ppc = std::min(npoly, 16);
-    pg.ppn = std::min(kGmacTile / pg.ppc, 16);
-    const int npg = (npoly + pg.ppc - 1) / pg.ppc;
-    dim3 g(((N / 2 + pg.ppn - 1) / pg.ppn) * npg, E);
-    FG_CHECK(g.x < (1u << 31), FG_EINVAL, "group_mac: grid too large");
-    const size_t sm = (size_t)pg.nsrc * kGmacTile * 16 + (size_t)pg.nterm * pg.ppn * 16;
-    double src_limbs = 0;
-    for (const auto &gs : srcs) src_limbs += gs.u ? E : level + 1;
-    KTimer kt(ctx, "group_mac",
-              (src_limbs * npoly + (double)pg.nterm * E +
-               (double)X * npoly * E * (accumulate ? 2 : 1)) * N * 8);
-    // raised once per process and size (not a stream operation, and kept out
-    // of the launches a CUDA graph capture records)
-    static size_t sm_set[4] = {48 * 1024, 48 * 1024, 48 * 1024, 48 * 1024};
-    const int v = (ctx->tune.gmac_regs ? 1 : 0) + (ctx->tune.kara ? 2 : 0);
-    auto kern = v == 0 ? k_group_mac<2, false> : v == 1 ? k_group_mac<3, false>
-              : v == 2 ? k_group_mac<2, true> : k_group_mac<3, true>;
-    if (sm > sm_set[v]) {
-        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        sm_set[v] = sm;
-    }
-    kern<<<g, G * kGmacTile, sm, ctx->stream>>>(pg, ncol, level, E, ls, ctx->log_n, ctx->d_pmodq,
-                                                ctx->d_primes, ctx->nq);
-    check_launch("group_mac");
 }
 
 // With ctx->tune.ks_cols = 2 the columns are split over two launches, so

@@ -56,7 +56,8 @@ std::vector<int> iota(int n, int start = 0)
 
 // put one encoded mask of the plan on the device over q_0..q_level and the
 // special primes (the latter lifted from limb 0: every mask coefficient is
-// below q_0 / 2 in magnitude), NTT domain, Montgomery form: [E][N]
+// below q_0 / 2 in magnitude), NTT domain, Montgomery form, each word in the
+// split halves its products take, and times P for kept values: [E][N]
 void upload_mask(fg_ctx *ctx, MaskC &m, const u64 *coeffs_host_or_dev)
 {
     const int N = ctx->n, nl = m.level + 1, E = ctx->ext(m.level);
@@ -68,7 +69,7 @@ void upload_mask(fg_ctx *ctx, MaskC &m, const u64 *coeffs_host_or_dev)
     for (int i = 0; i < E; i++) pid[i] = ctx->ext_prime(m.level, i);
     kern::LimbSet s{m.d, E, E, 1, pid};
     kern::ntt_fwd(ctx, s, s);
-    kern::to_mont(ctx, m.d, E, pid);
+    kern::to_mont(ctx, m.d, E, pid, true, m.kept);
 }
 
 void encode_mask(const fg_ctx *ctx, const MaskC &m, u64 *out)
@@ -91,6 +92,11 @@ static void finish_plan(fg_ctx *ctx, fg_plan *pl, bool no_encode)
 {
     const int N = ctx->n, F = pl->F, Fp = pl->Fp;
     const int nm = (int)pl->masks.size();
+    for (const GroupC &g : pl->groups)
+        for (const TermC &tm : g.terms) pl->masks[tm.mask].kept |= tm.k == 0;
+    for (const GroupC &g : pl->groups)   // a mask belongs to one term
+        for (const TermC &tm : g.terms)
+            FG_CHECK(pl->masks[tm.mask].kept == (tm.k == 0), FG_EINVAL, "mask shared by kept and rotated values");
     if (no_encode) {   // timing-only plan: zero masks, no host encoding
         for (MaskC &m : pl->masks) {
             const size_t bytes = (size_t)ctx->ext(m.level) * N * 8;
@@ -623,8 +629,7 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             u64 *tmp = acc_new;
             for (int k : pl->comb_rots) {
                 kern::modup(ctx, bufA[0], LS, Fp, l1, digits);
-                kern::rotate_mac(ctx, keys->get(((k % M) + M) % M), bufA[0], LS, Fp, l1, digits,
-                                 {{tmp, nullptr}}, LS);
+                kern::rotate(ctx, keys->get(((k % M) + M) % M), bufA[0], LS, Fp, l1, digits, tmp, LS);
                 kern::add(ctx, bufA[0], tmp, bufA[0], Fp * 2 * LS, pid_l1);
             }
         }
@@ -648,7 +653,7 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             std::map<std::pair<int, int>, std::vector<const TermC *>> by_src;
             for (const TermC &tm : g.terms) by_src[{tm.src, tm.k}].push_back(&tm);
             // sources per launch: the group's sources split evenly over the
-            // fewest launches within the program limits of k_group_mac (the
+            // fewest launches within the limits of group_mac (the
             // key-switch outputs of one launch are held at once)
             const int n_src = (int)by_src.size();
             const int n_launch = std::max({1, (n_src + kern::kGmacSrc - 1) / kern::kGmacSrc,
@@ -660,10 +665,8 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             std::vector<kern::Dest> terms;
             std::vector<int> tdest;
             bool first_flush = true;
-            std::vector<int> dest_terms(X, 0);   // terms per output since the last flush
             auto add_source = [&](const u64 *u, const u64 *lane, uint32_t galois,
                                   const std::vector<const TermC *> &ts) {
-                for (const TermC *tm : ts) dest_terms[out_index(tm->dst)]++;
                 kern::GroupSource gs{u, lane, galois, (int)terms.size(), 0};
                 for (const TermC *tm : ts) {
                     terms.push_back({nullptr, pl->masks[tm->mask].d});
@@ -686,9 +689,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             auto flush = [&]() {
                 issue_pending();
                 if (srcs.empty()) return;
-                // outputs in slices of at most 64 (the program's output table)
-                for (int x0 = 0; x0 < X; x0 += 64) {
-                    const int xn = std::min(64, X - x0);
+                // outputs in even slices of at most kGmacOut
+                const int n_sl = (X + kern::kGmacOut - 1) / kern::kGmacOut;
+                for (int sl = 0; sl < n_sl; sl++) {
+                    const int x0 = X * sl / n_sl, xn = X * (sl + 1) / n_sl - x0;
                     std::vector<kern::GroupSource> ss;
                     std::vector<kern::Dest> tt;
                     std::vector<int> td;
@@ -714,18 +718,14 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
                 srcs.clear();
                 terms.clear();
                 tdest.clear();
-                std::fill(dest_terms.begin(), dest_terms.end(), 0);
             };
-            auto needs_flush = [&](const std::vector<const TermC *> &ts) {
-                bool full = (int)srcs.size() >= per_launch ||
-                            (int)(terms.size() + ts.size()) > kern::kGmacTerms;
-                for (const TermC *tm : ts) full |= dest_terms[out_index(tm->dst)] >= 255;
-                return full;
+            auto full = [&](size_t more) {
+                return (int)srcs.size() >= per_launch || terms.size() + more > (size_t)kern::kGmacTerms;
             };
             // kept values first (no key switching)
             for (auto &kv : by_src)
                 if (kv.first.second == 0) {
-                    if (needs_flush(kv.second)) flush();
+                    if (full(kv.second.size())) flush();
                     add_source(nullptr, (*in)[kv.first.first], 0, kv.second);
                 }
             int cur = -1, used = 0;
@@ -733,7 +733,7 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
                 const int a = rk.first, k = rk.second;
                 auto it = by_src.find({a, k});
                 if (it == by_src.end()) continue;
-                if (needs_flush(it->second)) {
+                if (full(it->second.size())) {
                     flush();
                     used = 0;
                 }

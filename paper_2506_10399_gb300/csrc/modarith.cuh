@@ -126,6 +126,19 @@ __device__ __forceinline__ void mac_kara(u64 &a0, u64 &k, u64 &a2, u64 v, u64 m)
         : "r"(v0), "r"(v1), "r"(m0), "r"(m1), "r"(vs), "r"(ms));
 }
 
+// redc in two 32-bit steps, for q below 2^46 (S = hi 2^64 + lo <
+// q 2^64): each step adds the multiple of q that clears 32 low bits.  Six
+// multiplications where redc takes nine.
+__device__ __forceinline__ u64 redc46(u64 hi, u64 lo, const PrimeC &P)
+{
+    const u32 q0 = (u32)P.q, q1 = (u32)(P.q >> 32), n = (u32)P.qneg;
+    const u32 m0 = (u32)lo * n;
+    const u64 y = (u64)m0 * q1 + (lo >> 32) + (((u64)m0 * q0 + (u32)lo) >> 32);   // < 2^47
+    const u32 m1 = (u32)y * n;
+    const u64 z = (u64)m1 * q1 + (y >> 32) + (((u64)m1 * q0 + (u32)y) >> 32);
+    return reduce2(z + hi, P.q);
+}
+
 // (A0 + A1 2^23 + A2 2^46) R^-1 mod q.  The sum S = A0 + A1 2^23 + A2 2^46
 // of T < 2^16 products of reduced factors is below T q^2, so its high word
 // is below T q (q / 2^64) < q / 4 for q < 2^46: Montgomery's condition
@@ -139,7 +152,7 @@ __device__ __forceinline__ u64 fold_split(u64 a0, u64 a1, u64 a2, const PrimeC &
     t = a2 << 46;
     lo += t;
     hi += lo < t;
-    return redc(hi, lo, P);
+    return redc46(hi, lo, P);
 }
 
 __device__ __forceinline__ u64 fold_kara(u64 a0, u64 k, u64 a2, const PrimeC &P)
@@ -152,6 +165,13 @@ __device__ __forceinline__ u64 fold_kara(u64 a0, u64 k, u64 a2, const PrimeC &P)
 // 8 terms (A1 takes two products a term) before they are folded into a
 // 128-bit total.
 __device__ __forceinline__ u64 split30(u64 v) { return (v & 0x3FFFFFFF) | ((v >> 30) << 32); }
+
+// a word of prime q in the halves its products take, and back
+__device__ __forceinline__ u64 split_word(u64 v, u64 q) { return q < (1ull << 46) ? split23(v) : split30(v); }
+__device__ __forceinline__ u64 join_word(u64 s, u64 q)
+{
+    return (u64)(u32)s + (q < (1ull << 46) ? s >> 32 << 23 : s >> 32 << 30);
+}
 
 // (hi, lo) += A0 + A1 2^30 + A2 2^60
 __device__ __forceinline__ void fold30(u64 &hi, u64 &lo, u64 a0, u64 a1, u64 a2)
