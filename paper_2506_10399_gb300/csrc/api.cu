@@ -125,6 +125,24 @@ void *fg_ctx::buf(const std::string &name0, size_t bytes)
     return p;
 }
 
+int *fg_ctx::wait_error()
+{
+    if (!wait_err) {
+        CUDA_TRY(cudaHostAlloc(&wait_err, sizeof(int), cudaHostAllocMapped));
+        *wait_err = 0;
+    }
+    int *d = nullptr;
+    CUDA_TRY(cudaHostGetDevicePointer(&d, wait_err, 0));
+    return d;
+}
+
+void fg_ctx::check_waits()
+{
+    if (!wait_err || !*(volatile int *)wait_err) return;
+    *wait_err = 0;
+    throw fg_error(FG_ETIMEOUT, "a kernel's bounded wait ran out");
+}
+
 extern "C" int fg_ctx_release_workspace(fg_ctx *ctx)
 {
     if (!ctx) return FG_EINVAL;
@@ -622,6 +640,7 @@ int fg_ctx_destroy(fg_ctx *ctx)
     for (auto &kv : ctx->modup_scale_tabs) cudaFree(kv.second);
     for (auto &kv : ctx->moddown_scale_tabs) cudaFree(kv.second);
     for (auto &kv : ctx->ws) cudaFree(kv.second.first);
+    if (ctx->wait_err) cudaFreeHost(ctx->wait_err);
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     if (ctx->batch.exec) cudaGraphExecDestroy(ctx->batch.exec);
     for (cudaStream_t st : ctx->pool) cudaStreamDestroy(st);

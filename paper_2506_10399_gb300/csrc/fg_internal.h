@@ -194,6 +194,12 @@ struct fg_ctx {
         int64_t launches = 0;
     } batch;
 
+    // set by a kernel whose bounded wait ran out (page-locked, read by the
+    // host after a synchronisation)
+    int *wait_err = nullptr;
+    int *wait_error();      // its device address
+    void check_waits();     // throws FG_ETIMEOUT when it is set, and clears it
+
     int L() const { return nq - 1; }
     int ext(int level) const { return level + 1 + np; }
     int n_digits(int level) const { return (level + 1 + alpha - 1) / alpha; }
@@ -239,6 +245,18 @@ struct MaskC {
     u64 *d = nullptr;             // [E][N] NTT domain, Montgomery form, split halves (split_word)
 };
 
+// the combination's constants for the tensor cores (comb.cu)
+struct CombPlan {
+    int dc = 0;                 // 8-bit digits of the constants; 0: not available
+    int nj = 0, kb_all = 0;     // blocks of 16 outputs, of 16 columns
+    int corr_blocks = 0;        // blocks of 64 columns
+    void *dig = nullptr, *limb = nullptr;
+    u64 *corr = nullptr;
+    std::vector<int> da;        // 8-bit digits of an input word, by limb
+    void build(const fg_ctx &ctx, const std::vector<i64> &c, int F, int Fp, int level);
+    void release();
+};
+
 struct fg_plan {
     fg_ctx *ctx = nullptr;
     int N = 0, M = 0, t = 1, B = 0, V = 0, F = 0, Fp = 0;
@@ -250,6 +268,7 @@ struct fg_plan {
     std::vector<GroupC> groups;
     std::vector<MaskC> masks;
     u64 *d_comb = nullptr;                 // t == 1: [in_level+1][F][Fp] Montgomery constants
+    CombPlan comb;                         // t == 1: the same constants as 8-bit digits
     int max_lanes = 1;
     int n_copies = 0;                      // Inter-CA: neighbour copies (masks 0..n_copies-1)
 };
@@ -305,6 +324,11 @@ void expand_uniform(fg_ctx *ctx, cudaStream_t st, u64 *ct, size_t ct_pitch, cons
 // X: [F][2][level+1][N], consts: [level+1][F][Fp] Montgomery form, Z limb stride z_ls
 void comb_const_mac(fg_ctx *ctx, const u64 *X, int F, int Fp, int level, const u64 *consts,
                     u64 *Z, int z_ls, int fb = 0, int fe = -1, bool accumulate = false);
+// the plan's combination of columns fb..fe-1, on the tensor cores where columns
+// x blocks of 8 outputs >= kCombMmaMin x blocks of 16 outputs
+constexpr int kCombMmaMin = 40;
+void combine(fg_ctx *ctx, const fg_plan *pl, const u64 *X, u64 *Z, int z_ls, int fb = 0, int fe = -1,
+             bool accumulate = false);
 // rescale by q_level, coefficient domain, npoly polys with limb strides
 void rescale_coef(fg_ctx *ctx, const u64 *in, int in_ls, u64 *out, int out_ls, int npoly,
                   int level);

@@ -136,6 +136,7 @@ static void finish_plan(fg_ctx *ctx, fg_plan *pl, bool no_encode)
         }
         CUDA_TRY(cudaMalloc(&pl->d_comb, h.size() * 8));
         CUDA_TRY(cudaMemcpy(pl->d_comb, h.data(), h.size() * 8, cudaMemcpyHostToDevice));
+        pl->comb.build(*ctx, pl->comb_consts, F, Fp, l0);
     }
 }
 
@@ -203,6 +204,7 @@ int fg_plan_destroy(fg_plan *plan)
     if (plan->ctx) cudaStreamSynchronize(plan->ctx->stream);
     for (auto &m : plan->masks) cudaFree(m.d);
     cudaFree(plan->d_comb);
+    plan->comb.release();
     delete plan;
     return FG_OK;
 }
@@ -565,7 +567,7 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             u64 *Zc = (u64 *)ctx->buf("comb_z", (size_t)Fp * 2 * nl0 * N * 8);
             CUDA_TRY(cudaMemsetAsync(acc, 0, lane_w * 8, ctx->stream));
             for (int k = 0; k < pl->n_copies; k++) {
-                kern::comb_const_mac(ctx, X + (size_t)k * F * 2 * nl0 * N, F, Fp, l0, pl->d_comb, Zc, nl0);
+                kern::combine(ctx, pl, X + (size_t)k * F * 2 * nl0 * N, Zc, nl0);
                 kern::rescale_coef(ctx, Zc, nl0, bufA[0], LS, Fp * 2, l0);
                 kern::LimbSet z{bufA[0], LS, LS, Fp * 2, pid_l1};
                 kern::ntt_fwd(ctx, z, z);
@@ -584,7 +586,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             kern::copy_limbs(ctx, acc, LS, o, nlo, Fp * 2, nlo);
             if (o != out_cts)
                 CUDA_TRY(cudaMemcpyAsync(out_cts, o, out_w * 8, cudaMemcpyDeviceToHost, ctx->stream));
-            if (sync) CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+            if (sync) {
+                CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+                ctx->check_waits();
+            }
             if (out_level) *out_level = level;
             return;
         }
@@ -600,10 +605,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
                     if (seed)
                         kern::expand_uniform(ctx, ctx->stream, const_cast<u64 *>(X) + fb * ct_w, ct_w,
                                              c0s + fb * c0_w, fe - fb, nl0, *seed, (u64)fb);
-                    kern::comb_const_mac(ctx, X, F, Fp, l0, pl->d_comb, Zc, nl0, fb, fe, c > 0);
+                    kern::combine(ctx, pl, X, Zc, nl0, fb, fe, c > 0);
                 }
             } else {
-                kern::comb_const_mac(ctx, X, F, Fp, l0, pl->d_comb, Zc, nl0);
+                kern::combine(ctx, pl, X, Zc, nl0);
             }
             inputs_read();
             kern::rescale_coef(ctx, Zc, nl0, bufA[0], LS, Fp * 2, l0);
@@ -783,7 +788,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
         kern::copy_limbs(ctx, acc, LS, o, nlo, Fp * 2, nlo);
         if (o != out_cts)
             CUDA_TRY(cudaMemcpyAsync(out_cts, o, out_w * 8, cudaMemcpyDeviceToHost, ctx->stream));
-        if (sync) CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if (sync) {
+            CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+            ctx->check_waits();
+        }
         if (out_level) *out_level = level;
     }
 }
@@ -1074,6 +1082,7 @@ static int layer_batch(fg_ctx *ctx, const fg_keys *keys, const fg_plan *const *p
         batch_body(ctx, keys, plans, n, in_cts, out_cts, o, args, out_levels, streams_used);
         CUDA_TRY(cudaStreamSynchronize(ctx->stream));
         ctx->stream = home;
+        ctx->check_waits();
     } catch (const fg_error &e) {
         ctx->stream = home;
         ctx->err = e.what();
