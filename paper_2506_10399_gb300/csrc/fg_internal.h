@@ -96,8 +96,8 @@ struct Tune {
     int ntt_rows = 8;      // N = 2^16 NTT pass B: rows per CTA (8 or 16)
     int ntt_tw = 0;        // N = 2^16 NTT twiddles: 0 = held in registers per round (3 CTAs of
                            // 256 threads per SM), 1 = loaded where used (4 per SM)
-    int ks_split = 0;      // key switch registers: 0 = launch bounds by digit count, 1 = one CTA per
-                           // SM fewer, 2 = key words parked in shared memory (one CTA more)
+    int ks_split = 0;      // key switch registers: 0 = CTAs per SM by digit count, 1 = one fewer,
+                           // 2 = one more
     int ks_cols = 1;       // key switch: launches the columns are split over (1 or 2)
     int modup_fused = 1;   // N = 2^16 ModUp: 1 = conversion fused into the digits' first NTT pass
     int moddown_fused = 0; // N = 2^16 ModDown + rescale: 1 = conversion fused into the first NTT pass
@@ -359,6 +359,9 @@ constexpr int kGmacTerms = 300;
 void group_mac(fg_ctx *ctx, const std::vector<GroupSource> &srcs, const std::vector<Dest> &terms,
                const std::vector<int> &term_dest, const std::vector<u64 *> &outs, bool accumulate,
                int ncol, int level, int ls);
+// the same for up to 24 rotations in one launch, P phi_r(c0) only when add_c0
+void ks_launch(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::vector<u64 *> &us, const u64 *lane,
+               int ls, int ncol, int level, const u64 *digits, bool add_c0);
 // key-switch outputs u_r = sum_d D_d(sigma_r) evk_r + P phi_r(c0) of several
 // rotations r of one lane (extended basis, NTT domain, [ncol][2][E][N] each)
 void ks_multi(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::vector<u64 *> &us,

@@ -66,16 +66,6 @@ __device__ __forceinline__ void cp_async16(u64 *smem, const u64 *gmem)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 
-// a + x y.  (Between the branches of the inner loop the carry-chained pairs of
-// mac_split stayed two multiplications each and plain C sums became three
-// instructions; this form counts one multiplication.)
-__device__ __forceinline__ u64 mad_wide(u32 x, u32 y, u64 a)
-{
-    u64 p;
-    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(x), "r"(y));
-    return a + p;
-}
-
 // The warp's sums over one stage's sources for outputs bit 0..XS-1.  SMALL:
 // primes below 2^46, a[d][p] = (A0, K, A2) of mac_kara, at most 2^16 terms.
 // Otherwise 30-bit halves, a[d][p] = (A0, A1, A2) of mac_split with x3[d][p]

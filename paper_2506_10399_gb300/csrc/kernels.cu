@@ -402,9 +402,7 @@ k_modup_ntt16_a(const u64 *__restrict__ y, int nl, u64 *digits, int beta, int E,
 #pragma unroll
         for (int k = 0; k < NMAX; k++)
             if (k < T.n_in) mac_split(a0, a1, a2, split30(src[k][idx]), hm_[k]);
-        u64 hi = 0, lo = 0;
-        fold30(hi, lo, a0, a1, a2);
-        v[m] = redc(hi, lo, P);
+        v[m] = reduce30<NMAX>(a0, a1, a2, P);
     }
     __syncthreads();   // stw
     u64 *d = digits + (((size_t)f * beta + dg) * E + T.out_l[t]) * 65536 + c0;
@@ -757,15 +755,6 @@ __global__ void k_scalar(const u64 *a, u64 *c, const Batch bt, const PrimeC *__r
         c[off + x] = shoup_mul(a[off + x], w, ws, q);
 }
 
-// automorphism X -> X^g in the bit-reversed NTT order:
-// out[j] = a[brv(((2 brv(j) + 1) g mod 2N - 1) / 2)]
-__device__ __forceinline__ int auto_src(int j, uint32_t g, int log_n)
-{
-    uint32_t r = __brev((uint32_t)j) >> (32 - log_n);
-    uint32_t e = ((2 * r + 1) * g) & ((2u << log_n) - 1);
-    return (int)(__brev((e - 1) >> 1) >> (32 - log_n));
-}
-
 __global__ void k_automorphism(const u64 *a, u64 *c, int nlimbs, uint32_t g, int log_n)
 {
     const int N = 1 << log_n;
@@ -973,9 +962,7 @@ __device__ __forceinline__ u64 conv_point(const ConvTab &T, const u64 *y, int t,
     // centred conversion: c B subtracted (c <= 7: the product adds below
     // 2^34 to the partial sums, within the 8-term bound for K <= 7)
     if (c) mac_split(a0, a1, a2, (u64)c, T.negb[t]);
-    u64 hi = 0, lo = 0;
-    fold30(hi, lo, a0, a1, a2);
-    return redc(hi, lo, P);
+    return reduce30<NMAX>(a0, a1, a2, P);
 }
 
 // returns the number of inputs y_k above b_k / 2: taking those as y_k - b_k
@@ -1042,16 +1029,7 @@ k_moddown_conv(const u64 *__restrict__ u, int E, u64 *conv, int nl,
     }
 }
 
-// ------------------------------------------------------------------------
-// key switching inner product with the automorphism folded into the gather:
-//   u_p[f][i][x] = sum_d D_d[f][i][sigma_g(x)] * evk_g[d][p][i][x]
-// D_d limb i is the lane's own c1 limb when i belongs to digit d, else the
-// ModUp output.  The key (Montgomery form, [beta_L][2][nq+np][N]) is read
-// once per (x, i) and reused for every column.
-// ------------------------------------------------------------------------
-constexpr int kMaxBeta = 16;   // beta * p^2 < p * 2^64 needs beta * p < 2^64: p < 2^60
-
-// Each thread owns two adjacent slots x, x+1 (16-byte accesses).  In the
+// A thread that owns two adjacent slots x, x+1 makes 16-byte accesses.  In the
 // bit-reversed NTT order the automorphism maps every aligned pair {x, x+1}
 // onto an aligned pair {2m, 2m+1}, so the gather is one 16-byte load plus a
 // swap when sigma(x) is odd.
@@ -1059,122 +1037,6 @@ __device__ __forceinline__ ulonglong2 gather_pair(const u64 *limb, int m2, bool 
 {
     const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(limb)[m2 >> 1];
     return swap ? make_ulonglong2(v.y, v.x) : v;
-}
-
-// Several rotations of one lane in one launch: blockIdx.y picks the rotation
-// and blockIdx.z the limb, so the CTAs of one limb run together and the
-// lane's digits of that limb (ncol * beta limbs) are read from HBM once and
-// gathered again from L2 by the other rotations.
-constexpr int kKsMulti = 24;
-struct KsSet {
-    int n;
-    const u64 *key[kKsMulti];
-    uint32_t g[kKsMulti];
-    u64 *u[kKsMulti];
-};
-
-// With pmodq given, part 0 also receives P phi_g(c0) on the limbs of Q
-// (P mod q_i and its Shoup companion at pmodq[2i], pmodq[2i+1]), so that
-// ModDown of u is Rot(c) itself: ModDown(A + P B) = ModDown(A) + B exactly.
-// LESS: CTAs per SM one fewer than the default bound (more registers per
-// thread, fewer spills, lower occupancy); a tuning choice of the batched form.
-constexpr int ks_min_blocks(int beta, int less)
-{
-    return (beta <= 4 ? 4 : beta <= 5 ? 3 : 2) - less > 0 ? (beta <= 4 ? 4 : beta <= 5 ? 3 : 2) - less : 1;
-}
-
-// KSM: the thread's split key words are parked in shared memory (its own
-// 2 x BETA entries, no sharing, so no barrier) instead of registers, which
-// frees about 40 registers for one more CTA per SM; a tuning choice.
-template <int BETA, int LESS, bool KSM>
-__global__ void __launch_bounds__(256, KSM ? (BETA <= 4 ? 5 : 4) : ks_min_blocks(BETA, LESS))
-k_ks_ip(const KsSet ks, int KL, const u64 *__restrict__ lane, int ls,
-        const u64 *__restrict__ digits, int ncol, int level, int E, int alpha, int nq,
-        int log_n, const PrimeC *__restrict__ primes, const u64 *__restrict__ pmodq)
-{
-    extern __shared__ ulonglong2 kpark[];   // KSM: [BETA][2][blockDim.x]
-    const int N = 1 << log_n;
-    const int rot = blockIdx.y, i = blockIdx.z;
-    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (x >= N) return;
-    const u64 *key = ks.key[rot];
-    u64 *u = ks.u[rot];
-    const int pi = i <= level ? i : nq + (i - level - 1);
-    const PrimeC P = primes[pi];
-    const int sx = auto_src(x, ks.g[rot], log_n);
-    const bool swap = sx & 1;
-    const int own = i <= level ? i / alpha : -1;
-    // Sums of BETA products of words below 2^60: with 30-bit halves (keys
-    // split once per thread, each gathered digit word once for its two
-    // products) the three 64-bit partial sums hold up to 8 products per
-    // term; more digits take the 128-bit sums.  The total, below
-    // BETA 2^60 q, keeps its high word below q for the Montgomery step.
-    constexpr bool SPLIT = BETA <= 8;
-    ulonglong2 kb[KSM ? 1 : BETA], ka[KSM ? 1 : BETA];
-#pragma unroll
-    for (int d = 0; d < BETA; d++) {
-        ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(key + (((size_t)d * 2 + 0) * KL + pi) * N + x);
-        ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(key + (((size_t)d * 2 + 1) * KL + pi) * N + x);
-        if (SPLIT) {
-            b = make_ulonglong2(split30(b.x), split30(b.y));
-            a = make_ulonglong2(split30(a.x), split30(a.y));
-        }
-        if (KSM) {
-            kpark[(d * 2 + 0) * blockDim.x + threadIdx.x] = b;
-            kpark[(d * 2 + 1) * blockDim.x + threadIdx.x] = a;
-        } else {
-            kb[KSM ? 0 : d] = b;
-            ka[KSM ? 0 : d] = a;
-        }
-    }
-    auto KB = [&](int d) { return KSM ? kpark[(d * 2 + 0) * blockDim.x + threadIdx.x] : kb[KSM ? 0 : d]; };
-    auto KA = [&](int d) { return KSM ? kpark[(d * 2 + 1) * blockDim.x + threadIdx.x] : ka[KSM ? 0 : d]; };
-    for (int f = 0; f < ncol; f++) {
-        ulonglong2 r0, r1;
-        if (SPLIT) {
-            u64 a[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int d = 0; d < BETA; d++) {
-                const u64 *limb = d == own ? lane + (((size_t)f * 2 + 1) * ls + i) * N
-                                           : digits + (((size_t)f * BETA + d) * E + i) * N;
-                ulonglong2 v = gather_pair(limb, sx, swap);
-                v = make_ulonglong2(split30(v.x), split30(v.y));
-                const ulonglong2 b = KB(d), kk = KA(d);
-                mac_split(a[0], a[1], a[2], v.x, b.x);
-                mac_split(a[3], a[4], a[5], v.y, b.y);
-                mac_split(a[6], a[7], a[8], v.x, kk.x);
-                mac_split(a[9], a[10], a[11], v.y, kk.y);
-            }
-            u64 h[4] = {0, 0, 0, 0}, l[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int c = 0; c < 4; c++) fold30(h[c], l[c], a[3 * c], a[3 * c + 1], a[3 * c + 2]);
-            r0 = make_ulonglong2(redc(h[0], l[0], P), redc(h[1], l[1], P));
-            r1 = make_ulonglong2(redc(h[2], l[2], P), redc(h[3], l[3], P));
-        } else {
-            u64 h0 = 0, l0 = 0, h1 = 0, l1 = 0, h2 = 0, l2 = 0, h3 = 0, l3 = 0;
-#pragma unroll
-            for (int d = 0; d < BETA; d++) {
-                const u64 *limb = d == own ? lane + (((size_t)f * 2 + 1) * ls + i) * N
-                                           : digits + (((size_t)f * BETA + d) * E + i) * N;
-                const ulonglong2 v = gather_pair(limb, sx, swap);
-                const ulonglong2 b = KB(d), kk = KA(d);
-                mac128(h0, l0, v.x, b.x);
-                mac128(h1, l1, v.y, b.y);
-                mac128(h2, l2, v.x, kk.x);
-                mac128(h3, l3, v.y, kk.y);
-            }
-            r0 = make_ulonglong2(redc(h0, l0, P), redc(h1, l1, P));
-            r1 = make_ulonglong2(redc(h2, l2, P), redc(h3, l3, P));
-        }
-        if (pmodq && i <= level) {
-            const ulonglong2 c0 = gather_pair(lane + (((size_t)f * 2) * ls + i) * N, sx, swap);
-            const u64 pw = pmodq[2 * i], pws = pmodq[2 * i + 1];
-            r0.x = add_mod(r0.x, shoup_mul(c0.x, pw, pws, P.q), P.q);
-            r0.y = add_mod(r0.y, shoup_mul(c0.y, pw, pws, P.q), P.q);
-        }
-        *reinterpret_cast<ulonglong2 *>(u + (((size_t)f * 2 + 0) * E + i) * N + x) = r0;
-        *reinterpret_cast<ulonglong2 *>(u + (((size_t)f * 2 + 1) * E + i) * N + x) = r1;
-    }
 }
 
 // ------------------------------------------------------------------------
@@ -1378,9 +1240,7 @@ k_moddown_ntt16_a(const u64 *__restrict__ ext, int E, u64 *w, int l, const ConvT
         for (int k = 0; k < NMAX; k++)
             if (k < T.n_in) mac_split(a0, a1, a2, split30(base[(size_t)T.in_l[k] * 65536 + idx]), hm_[k]);
         if (cc) mac_split(a0, a1, a2, (u64)cc, nb);
-        u64 hi = 0, lo = 0;
-        fold30(hi, lo, a0, a1, a2);
-        const u64 conv = redc(hi, lo, P);
+        const u64 conv = reduce30<NMAX>(a0, a1, a2, P);
         v[m] = sub_mod(add_mod(conv, shoup_mul(ol, pw, pws, P.q), P.q), ht, P.q);
     }
     __syncthreads();   // stw
@@ -1784,61 +1644,10 @@ void modup(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level, u64 *digit
     ntt_fwd(ctx, ds, ds);
 }
 
-// key-switch inner products of up to kKsMulti rotations of one lane (with
-// P phi(c0) folded in when add_c0 is set)
-static void ks_launch(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::vector<u64 *> &us,
-                      const u64 *lane, int ls, int ncol, int level, const u64 *digits, bool add_c0)
-{
-    const int N = ctx->n, E = ctx->ext(level), beta = ctx->n_digits(level);
-    FG_CHECK(beta <= kMaxBeta, FG_EINVAL, "too many key-switching digits");
-    FG_CHECK(!keys.empty() && keys.size() <= (size_t)kKsMulti && keys.size() == us.size(), FG_EINVAL,
-             "ks_launch: 1 to 24 rotations");
-    const int KL = ctx->nq + ctx->np;
-    KsSet ks;
-    memset(&ks, 0, sizeof(ks));
-    ks.n = (int)keys.size();
-    for (int r = 0; r < ks.n; r++) {
-        ks.key[r] = keys[r]->d;
-        ks.g[r] = keys[r]->galois;
-        ks.u[r] = us[r];
-    }
-    const u64 *pmodq = add_c0 ? ctx->d_pmodq : nullptr;
-    dim3 g1((N / 2 + 255) / 256, ks.n, E);
-    // digits and c0 once per launch, keys and outputs once per rotation
-    KTimer kt(ctx, "ks_ip", ((double)ncol * beta * E + (add_c0 ? (double)ncol * (level + 1) : 0) +
-                             (double)ks.n * (2.0 * beta * E + 2.0 * ncol * E)) * N * 8);
-#define FG_KS_CASE(B)                                                                          \
-    case B:                                                                                    \
-        if (ksm && B <= 6)                                                                     \
-            k_ks_ip<B, 0, (B <= 6)><<<g1, 256, (size_t)B * 2 * 256 * 16, ctx->stream>>>(         \
-                ks, KL, lane, ls, digits, ncol, level, E, ctx->alpha, ctx->nq, ctx->log_n,     \
-                ctx->d_primes, pmodq);                                                         \
-        else if (less)                                                                         \
-            k_ks_ip<B, (B <= 8 ? 1 : 0), false><<<g1, 256, 0, ctx->stream>>>(                   \
-                ks, KL, lane, ls, digits, ncol, level, E, ctx->alpha, ctx->nq, ctx->log_n,     \
-                ctx->d_primes, pmodq);                                                         \
-        else                                                                                   \
-            k_ks_ip<B, 0, false><<<g1, 256, 0, ctx->stream>>>(ks, KL, lane, ls, digits, ncol,   \
-                                                              level, E, ctx->alpha, ctx->nq,   \
-                                                              ctx->log_n, ctx->d_primes, pmodq); \
-        break;
-    const bool less = ctx->tune.ks_split == 1, ksm = ctx->tune.ks_split == 2;
-    switch (beta) {
-        FG_KS_CASE(1) FG_KS_CASE(2) FG_KS_CASE(3) FG_KS_CASE(4) FG_KS_CASE(5) FG_KS_CASE(6)
-        FG_KS_CASE(7) FG_KS_CASE(8) FG_KS_CASE(9) FG_KS_CASE(10) FG_KS_CASE(11) FG_KS_CASE(12)
-        FG_KS_CASE(13) FG_KS_CASE(14) FG_KS_CASE(15) FG_KS_CASE(16)
-    default: throw fg_error(FG_EINVAL, "too many key-switching digits");
-    }
-#undef FG_KS_CASE
-    check_launch("ks_ip");
-}
-
 void rotate(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, int level, const u64 *digits, u64 *out,
             int out_ls)
 {
     const int N = ctx->n, nl = level + 1, E = ctx->ext(level), beta = ctx->n_digits(level);
-    FG_CHECK(beta <= kMaxBeta, FG_EINVAL, "too many key-switching digits");
-    const int KL = ctx->nq + ctx->np;
     u64 *u = (u64 *)ctx->buf("ks_u", (size_t)ncol * 2 * E * N * 8);
     ks_launch(ctx, {&key}, {u}, lane, ls, ncol, level, digits, false);
     std::vector<int> pp(E);
@@ -1896,28 +1705,6 @@ void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out)
                                                                       ctx->np, ctx->nq,
                                                                       ctx->d_primes, ctx->n);
     check_launch("lift_special");
-}
-
-// With ctx->tune.ks_cols = 2 the columns are split over two launches, so
-// that the digits a limb's CTAs gather from L2 are half as many (the keys
-// are then read once per half).
-void ks_multi(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::vector<u64 *> &us,
-              const u64 *lane, int ls, int ncol, int level, const u64 *digits)
-{
-    const int E = ctx->ext(level), beta = ctx->n_digits(level), N = ctx->n;
-    const int parts = std::max(1, std::min(ctx->tune.ks_cols, ncol));
-    for (int h = 0; h < parts; h++) {
-        const int f0 = ncol * h / parts, f1 = ncol * (h + 1) / parts;
-        if (f1 == f0) continue;
-        for (size_t r0 = 0; r0 < keys.size(); r0 += kKsMulti) {
-            const size_t r1 = std::min(keys.size(), r0 + kKsMulti);
-            std::vector<u64 *> uh;
-            for (size_t r = r0; r < r1; r++) uh.push_back(us[r] + (size_t)f0 * 2 * E * N);
-            ks_launch(ctx, std::vector<const KeyDev *>(keys.begin() + r0, keys.begin() + r1), uh,
-                      lane + (size_t)f0 * 2 * ls * N, ls, f1 - f0, level,
-                      digits + (size_t)f0 * beta * E * N, true);
-        }
-    }
 }
 
 // ModDown + rescale at N = 2^16 with the conversion fused into w's first

@@ -126,33 +126,33 @@ __device__ __forceinline__ void mac_kara(u64 &a0, u64 &k, u64 &a2, u64 v, u64 m)
         : "r"(v0), "r"(v1), "r"(m0), "r"(m1), "r"(vs), "r"(ms));
 }
 
-// redc in two 32-bit steps, for q below 2^46 (S = hi 2^64 + lo <
-// q 2^64): each step adds the multiple of q that clears 32 low bits.  Six
-// multiplications where redc takes nine.
-__device__ __forceinline__ u64 redc46(u64 hi, u64 lo, const PrimeC &P)
+// a + x y.  (In places, between branches above all, the carry-chained pairs of
+// mac_split stayed two multiplications each and plain C sums became three
+// instructions; this form counts one multiplication.)
+__device__ __forceinline__ u64 mad_wide(u32 x, u32 y, u64 a)
 {
-    const u32 q0 = (u32)P.q, q1 = (u32)(P.q >> 32), n = (u32)P.qneg;
-    const u32 m0 = (u32)lo * n;
-    const u64 y = (u64)m0 * q1 + (lo >> 32) + (((u64)m0 * q0 + (u32)lo) >> 32);   // < 2^47
-    const u32 m1 = (u32)y * n;
-    const u64 z = (u64)m1 * q1 + (y >> 32) + (((u64)m1 * q0 + (u32)y) >> 32);
-    return reduce2(z + hi, P.q);
+    u64 p;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(x), "r"(y));
+    return a + p;
 }
 
-// (A0 + A1 2^23 + A2 2^46) R^-1 mod q.  The sum S = A0 + A1 2^23 + A2 2^46
-// of T < 2^16 products of reduced factors is below T q^2, so its high word
-// is below T q (q / 2^64) < q / 4 for q < 2^46: Montgomery's condition
-// S < q 2^64 holds without reducing the high word first.
+// (A0 + A1 2^23 + A2 2^46) R^-1 mod q, R = 2^64, by Montgomery steps of 23, 23
+// and 18 bits on the partial sums themselves: each step adds the multiple of
+// q = q0 + q1 2^23 that clears the low bits of one sum and carries the rest
+// into the next, so that the 128-bit total is never formed (27 instructions
+// against 60 with it, and nine products either way).  The total S of T < 2^16
+// products of reduced factors is below T q^2, so S / 2^64 < T q (q / 2^64) < q
+// / 4 for q < 2^46, and the result, S / 2^64 plus less than q, needs one
+// subtraction.  The sums stay below 2^62 + 2^46 + 2^41.
 __device__ __forceinline__ u64 fold_split(u64 a0, u64 a1, u64 a2, const PrimeC &P)
 {
-    u64 lo = a0, hi = (a1 >> 41) + (a2 >> 18);
-    u64 t = a1 << 23;
-    lo += t;
-    hi += lo < t;
-    t = a2 << 46;
-    lo += t;
-    hi += lo < t;
-    return redc46(hi, lo, P);
+    const u32 q0 = (u32)P.q & 0x7FFFFF, q1 = (u32)(P.q >> 23), n = (u32)P.qneg;
+    const u32 m0 = (u32)a0 * n & 0x7FFFFF;
+    a1 = mad_wide(m0, q1, a1) + (mad_wide(m0, q0, a0) >> 23);
+    const u32 m1 = (u32)a1 * n & 0x7FFFFF;
+    a2 = mad_wide(m1, q1, a2) + (mad_wide(m1, q0, a1) >> 23);
+    const u32 m2 = (u32)a2 * n & 0x3FFFF;
+    return reduce2(mad_wide(m2, q1 << 5, mad_wide(m2, q0, a2) >> 18), P.q);
 }
 
 __device__ __forceinline__ u64 fold_kara(u64 a0, u64 k, u64 a2, const PrimeC &P)
@@ -186,6 +186,33 @@ __device__ __forceinline__ void fold30(u64 &hi, u64 &lo, u64 a0, u64 a1, u64 a2)
     hi += (lo < t) + (a2 >> 4);
 }
 
+// (A0 + A1 2^30 + A2 2^60) R^-1 mod q for q below 2^60, by Montgomery steps of
+// 30, 30 and 4 bits as in fold_split.  For sums of at most kRedc30 products of
+// 30-bit halves (A1 takes two a term): A1 plus two products of a step and a
+// carry stays below 14 2^60 + 2^35 < 2^64.  The total must be below q 2^64.
+constexpr int kRedc30 = 6;
+__device__ __forceinline__ u64 redc30(u64 a0, u64 a1, u64 a2, const PrimeC &P)
+{
+    const u32 q0 = (u32)P.q & 0x3FFFFFFF, q1 = (u32)(P.q >> 30), n = (u32)P.qneg;
+    const u32 m0 = (u32)a0 * n & 0x3FFFFFFF;
+    a1 = mad_wide(m0, q1, a1) + (mad_wide(m0, q0, a0) >> 30);
+    const u32 m1 = (u32)a1 * n & 0x3FFFFFFF;
+    a2 = mad_wide(m1, q1, a2) + (mad_wide(m1, q0, a1) >> 30);
+    const u32 m2 = (u32)a2 * n & 15;
+    return reduce2((mad_wide(m2, q0, a2) >> 4) + (mad_wide(m2, q1, 0) << 26), P.q);
+}
+
+// the same for sums of up to eight products: N of them
+template <int N>
+__device__ __forceinline__ u64 reduce30(u64 a0, u64 a1, u64 a2, const PrimeC &P)
+{
+    static_assert(N <= 8, "partial sums of 64 bits hold eight products of 30-bit halves");
+    if (N <= kRedc30) return redc30(a0, a1, a2, P);
+    u64 hi = 0, lo = 0;
+    fold30(hi, lo, a0, a1, a2);
+    return redc(hi, lo, P);
+}
+
 // Shoup product with a three-product quotient that skips the carries of the
 // low partial products: h = y_hi w'_hi + hi(y_lo w'_hi) + hi(y_hi w'_lo)
 // leaves out y_lo w'_lo and the low halves of the cross products, three
@@ -199,4 +226,13 @@ __device__ __forceinline__ u64 shoup_lazy4(u64 y, u64 w, u64 ws, u64 q)
     u64 h;
     asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(h) : "r"(y1), "r"(s1), "l"(c));
     return y * w - h * q;
+}
+
+// automorphism X -> X^g in the bit-reversed NTT order:
+// out[j] = a[brv(((2 brv(j) + 1) g mod 2N - 1) / 2)]
+__device__ __forceinline__ int auto_src(int j, uint32_t g, int log_n)
+{
+    uint32_t r = __brev((uint32_t)j) >> (32 - log_n);
+    uint32_t e = ((2 * r + 1) * g) & ((2u << log_n) - 1);
+    return (int)(__brev((e - 1) >> 1) >> (32 - log_n));
 }
