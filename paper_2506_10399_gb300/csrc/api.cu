@@ -585,6 +585,12 @@ int fg_ctx_create(const fg_params *prm, void *cuda_stream, fg_ctx **out)
             CUDA_TRY(cudaMemcpy(ctx->d_inv_rows, ir.data(), sizeof(ulonglong2) * KL * per, cudaMemcpyHostToDevice));
             ctx->table_bytes += 2 * sizeof(ulonglong2) * KL * per;
         }
+        if (ctx->log_n < 16) {
+            CUDA_TRY(cudaMalloc(&ctx->d_fwd_last, sizeof(ulonglong2) * KL * N));
+            CUDA_TRY(cudaMalloc(&ctx->d_inv_last, sizeof(ulonglong2) * KL * N));
+            ntt_last_tables(ctx);
+            ctx->table_bytes += 2 * sizeof(ulonglong2) * KL * N;
+        }
         // P mod q_i (Shoup) and the identity prime-index list
         std::vector<u64> pm(2 * ctx->nq);
         for (int i = 0; i < ctx->nq; i++) {
@@ -631,6 +637,8 @@ int fg_ctx_destroy(fg_ctx *ctx)
     cudaFree(ctx->d_inv);
     cudaFree(ctx->d_fwd_rows);
     cudaFree(ctx->d_inv_rows);
+    cudaFree(ctx->d_fwd_last);
+    cudaFree(ctx->d_inv_last);
     cudaFree(ctx->d_ninv);
     for (auto &kv : ctx->conv_tabs) cudaFree(kv.second);
     for (auto &kv : ctx->rescale_tabs) cudaFree(kv.second);

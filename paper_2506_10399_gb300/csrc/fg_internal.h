@@ -137,6 +137,10 @@ struct fg_ctx {
     // so that the 16 threads of a row read 16 consecutive entries
     void *d_fwd_rows = nullptr;       // ulonglong2 [nq+np][256][15][16]
     void *d_inv_rows = nullptr;
+    // N < 2^16: the twiddles of the transform's last register round, laid out
+    // [group of the round][group of elements] (see ntt.cu)
+    void *d_fwd_last = nullptr;       // ulonglong2 [nq+np][N]
+    void *d_inv_last = nullptr;
     u64 *d_ninv = nullptr;            // [nq+np][2] N^-1 and Shoup
     u64 *d_pmodq = nullptr;           // [nq][2] P mod q_i and Shoup
     std::vector<u64> h_qneg, h_r2, h_ones;
@@ -272,6 +276,9 @@ struct fg_plan {
     int max_lanes = 1;
     int n_copies = 0;                      // Inter-CA: neighbour copies (masks 0..n_copies-1)
 };
+
+// fills d_fwd_last and d_inv_last from d_fwd and d_inv (N < 2^16)
+void ntt_last_tables(fg_ctx *ctx);
 
 // ------------------------------------------------------------------ kernels
 namespace kern {

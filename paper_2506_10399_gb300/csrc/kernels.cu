@@ -7,22 +7,9 @@
 // column c is reduced modulo prime pidx[c] (pidx < 0: leave that limb).
 #include <cstdio>
 
-#include "fg_internal.h"
-#include "modarith.cuh"
+#include "ntt.cuh"
 
 namespace {
-
-constexpr int kPidxMax = 1024;
-
-struct Batch {
-    u64 *src;          // read from
-    u64 *dst;          // written to (may equal src)
-    int src_stride;    // limbs between rows
-    int dst_stride;
-    int per_row;
-    int rows;
-    int8_t pidx[kPidxMax];
-};
 
 Batch make_batch(u64 *src, int src_stride, u64 *dst, int dst_stride, int per_row, int rows,
                  const std::vector<int> &pidx)
@@ -50,92 +37,13 @@ inline void check_launch(const char *what, int kernels = 1)
 }
 
 // ------------------------------------------------------------------------
-// NTT: negacyclic, Cooley-Tukey forward with twiddles psi^brv(m+i) (natural
-// order in, bit-reversed order out: out[j] = a(psi^(2 brv(j) + 1))),
-// Gentleman-Sande inverse, Harvey's lazy butterflies.  N = N1 * N2 with
-// N1 = 2^s1: pass A runs stages 0..s1-1 on the N2 stride-N2 columns, pass B
-// runs the remaining stages inside each of the N1 contiguous rows.
+// NTT at N = 2^16 (smaller rings: ntt.cu): negacyclic, Cooley-Tukey forward
+// with twiddles psi^brv(m+i) (natural order in, bit-reversed order out: out[j]
+// = a(psi^(2 brv(j) + 1))), Gentleman-Sande inverse, Harvey's lazy butterflies.
+// N = 256 x 256: pass A runs stages 0..7 on the columns, pass B stages 8..15
+// inside the rows, each as two radix-16 register rounds (ct_round, gs_round)
+// with one shared-memory exchange.
 // ------------------------------------------------------------------------
-constexpr int kNttThreads = 256;
-constexpr int kColsA = 16;       // columns per CTA in pass A
-constexpr int kElemsB = 2048;    // elements per CTA in pass B
-
-__device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q2)
-{
-    X = X >= q2 ? X - q2 : X;               // X < 2q, Y < 4q in; both < 4q out
-    const u64 T = shoup_lazy(Y, w.x, w.y, q);
-    Y = X - T + q2;
-    X = X + T;
-}
-
-__device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, const ulonglong2 w, u64 q, u64 q2)
-{
-    const u64 U = X, V = Y;                 // both < 2q in and out
-    const u64 S = U + V;
-    X = S >= q2 ? S - q2 : S;
-    Y = shoup_lazy(U - V + q2, w.x, w.y, q);
-}
-
-// ------------------------------------------------------------------------
-// log N = 16: radix-16 rounds.  Every thread holds 16 elements in registers
-// for four stages, so each pass makes two shared-memory round trips
-// (N = 256 x 256; pass A on columns, pass B on rows).  For primes below
-// 2^47 the butterflies skip every conditional reduction and use the
-// three-product quotient without carries (shoup_lazy4, products in
-// [0, 4q)): forward values grow by at most 4q per stage (< 65q after 16
-// stages); inverse values are below 2^(k+1) q after k stages (< 2^64 for
-// q < 2^47); one reduction at the end restores [0, q).  Larger primes keep
-// Harvey's bounds (< 4q, < 2q).
-// ------------------------------------------------------------------------
-// tw(st, g): twiddle of group g at stage st (0..3) of the 16-point round
-template <bool LAZY, class TW>
-__device__ __forceinline__ void ct16(u64 (&v)[16], TW tw, u64 q, u64 q2)
-{
-#pragma unroll
-    for (int st = 0; st < 4; st++) {
-        const int h = 8 >> st;
-#pragma unroll
-        for (int m = 0; m < 16; m++) {
-            if ((m & h) == 0) {
-                const ulonglong2 w = tw(st, m >> (4 - st));
-                u64 X = v[m], Y = v[m + h];
-                if (LAZY) {
-                    const u64 T = shoup_lazy4(Y, w.x, w.y, q);
-                    v[m + h] = X - T + 4 * q;
-                    v[m] = X + T;
-                } else {
-                    X = X >= q2 ? X - q2 : X;
-                    const u64 T = shoup_lazy(Y, w.x, w.y, q);
-                    v[m + h] = X - T + q2;
-                    v[m] = X + T;
-                }
-            }
-        }
-    }
-}
-
-// k0: number of inverse stages already applied to these values (lazy bound 2^k0 q)
-template <bool LAZY, class TW>
-__device__ __forceinline__ void gs16(u64 (&v)[16], TW tw, u64 q, u64 q2, int k0)
-{
-#pragma unroll
-    for (int st = 3; st >= 0; st--) {
-        const int h = 8 >> st;
-        const u64 qb = LAZY ? (q << (k0 + 4 - st)) : q2;   // above the bound of V
-#pragma unroll
-        for (int m = 0; m < 16; m++) {
-            if ((m & h) == 0) {
-                const ulonglong2 w = tw(st, m >> (4 - st));
-                const u64 U = v[m], V = v[m + h];
-                const u64 S = U + V;
-                v[m] = LAZY ? S : (S >= q2 ? S - q2 : S);
-                v[m + h] = LAZY ? shoup_lazy4(U - V + qb, w.x, w.y, q)
-                                : shoup_lazy(U - V + qb, w.x, w.y, q);
-            }
-        }
-    }
-}
-
 // A round's 15 twiddles either held in registers for the whole round
 // (OD = false: loaded up front) or loaded where each stage uses them (OD =
 // true: fewer live registers, so more CTAs per SM).
@@ -177,13 +85,13 @@ __device__ __forceinline__ void fwd_a16_rounds(u64 (&v)[16], u64 *d, const ulong
     constexpr int N2 = 256;
     const u64 q2 = 2 * q;
     // stage st, group g at (1 << st) + g
-    ct16<LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[(r + 16 * m) * COLS + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[(16 * r + m) * COLS + c];
-    ct16<LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2);
 #pragma unroll
     for (int m = 0; m < 16; m++) d[(size_t)(16 * r + m) * N2 + c] = v[m];   // lazy
 }
@@ -232,7 +140,7 @@ __device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, cons
     u64 *drow = d + (size_t)r * 256;
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = drow[j + 16 * m];
-    ct16<LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2);
     u64 *srow = sm + r * kR16Row;
 #pragma unroll
     for (int m = 0; m < 16; m++) srow[pad16(j + 16 * m)] = v[m];
@@ -240,7 +148,7 @@ __device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, cons
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = srow[pad16(16 * j + m)];
     // row stages 12..15 from the row-blocked table (consecutive per row)
-    ct16<LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
                q, q2);
     ulonglong2 *o = reinterpret_cast<ulonglong2 *>(drow + 16 * j);
 #pragma unroll
@@ -284,7 +192,7 @@ __device__ __forceinline__ void inv_b16_body(const u64 *s, u64 *d, const ulonglo
         v[m] = a.x;
         v[m + 1] = a.y;
     }
-    gs16<LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
                q, q2, 0);
     u64 *srow = sm + r * kR16Row;
 #pragma unroll
@@ -292,7 +200,7 @@ __device__ __forceinline__ void inv_b16_body(const u64 *s, u64 *d, const ulonglo
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = srow[pad16(j + 16 * m)];
-    gs16<LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2, 4);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2, 4);
     u64 *drow = d + (size_t)r * 256;
 #pragma unroll
     for (int m = 0; m < 16; m++) drow[j + 16 * m] = v[m];   // lazy (< 2^9 q or < 2q)
@@ -328,13 +236,13 @@ __device__ __forceinline__ void inv_a16_body(u64 *d, const ulonglong2 *stw, u64 
     u64 v[16];
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = d[(size_t)(16 * r + m) * N2 + c];
-    gs16<LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2, 8);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2, 8);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[(16 * r + m) * COLS + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[(r + 16 * m) * COLS + c];
-    gs16<LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2, 12);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2, 12);
 #pragma unroll
     for (int m = 0; m < 16; m++) d[(size_t)(r + 16 * m) * N2 + c] = shoup_mul(v[m], ni, nis, q);
 }
@@ -408,260 +316,6 @@ k_modup_ntt16_a(const u64 *__restrict__ y, int nl, u64 *digits, int beta, int E,
     u64 *d = digits + (((size_t)f * beta + dg) * E + T.out_l[t]) * 65536 + c0;
     if (P.q < (1ull << 47)) fwd_a16_rounds<true, COLS, OD>(v, d, stw, P.q, sm);
     else fwd_a16_rounds<false, COLS, OD>(v, d, stw, P.q, sm);
-}
-
-// Stages are taken two at a time (radix-4 rounds: four elements, four
-// butterflies, one shared-memory round trip and one barrier per two
-// stages).  Within a sub-transform of 2^LS elements, a round on stages
-// (s, s+1) (s counted inside the sub-transform) works on element groups
-// {r, r + h/2, r + h, r + 3h/2} with h = 2^(LS-s-1), r = (i << (LS-s)) + j,
-// i = unit >> (LS-s-2), j = unit & (h/2 - 1); stage s uses twiddle index
-// 2^s + i, stage s+1 uses 2^(s+1) + 2i and 2^(s+1) + 2i + 1 (offset by the
-// sub-transform's position in the global stage numbering, see callers).
-
-template <int LOGN>
-__global__ void __launch_bounds__(kNttThreads)
-ntt_fwd_a(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ tw)
-{
-    constexpr int S1 = LOGN / 2, N = 1 << LOGN, N1 = 1 << S1, N2 = N >> S1;
-    constexpr int LC = 4;   // log2 kColsA
-    const int limb = blockIdx.y;
-    const int col = limb % bt.per_row, row = limb / bt.per_row;
-    const int pi = bt.pidx[col];
-    if (pi < 0) return;
-    extern __shared__ u64 sm[];
-    ulonglong2 *stw = reinterpret_cast<ulonglong2 *>(sm + N1 * kColsA);
-    const u64 q = primes[pi].q, q2 = 2 * q;
-    const ulonglong2 *twp = tw + (size_t)pi * N;
-    const u64 *src = bt.src + ((size_t)row * bt.src_stride + col) * N;
-    u64 *dst = bt.dst + ((size_t)row * bt.dst_stride + col) * N;
-    const int c0 = blockIdx.x * kColsA;
-    for (int i = threadIdx.x; i < N1; i += kNttThreads) stw[i] = twp[i];
-    for (int idx = threadIdx.x; idx < N1 * kColsA; idx += kNttThreads)
-        sm[idx] = src[(size_t)(idx >> LC) * N2 + c0 + (idx & (kColsA - 1))];
-    __syncthreads();
-    int s = 0;
-#pragma unroll
-    for (; s + 1 < S1; s += 2) {
-        const int lq = S1 - s - 2;   // log of h/2
-#pragma unroll 2
-        for (int b = threadIdx.x; b < (N1 / 4) * kColsA; b += kNttThreads) {
-            const int c = b & (kColsA - 1), u = b >> LC;
-            const int i = u >> lq, j = u & ((1 << lq) - 1);
-            const int r = (i << (lq + 2)) + j;
-            const ulonglong2 w1 = stw[(1 << s) + i];
-            const ulonglong2 w2 = stw[(2 << s) + 2 * i], w3 = stw[(2 << s) + 2 * i + 1];
-            u64 *p0 = sm + r * kColsA + c;
-            const int dq = (1 << lq) * kColsA;
-            u64 a0 = p0[0], a1 = p0[dq], a2 = p0[2 * dq], a3 = p0[3 * dq];
-            ct_bfly(a0, a2, w1, q, q2);
-            ct_bfly(a1, a3, w1, q, q2);
-            ct_bfly(a0, a1, w2, q, q2);
-            ct_bfly(a2, a3, w3, q, q2);
-            p0[0] = a0;
-            p0[dq] = a1;
-            p0[2 * dq] = a2;
-            p0[3 * dq] = a3;
-        }
-        __syncthreads();
-    }
-    if (s < S1) {   // odd stage count: last radix-2 stage (h = 1)
-        for (int b = threadIdx.x; b < (N1 / 2) * kColsA; b += kNttThreads) {
-            const int c = b & (kColsA - 1), i = b >> LC;
-            u64 *p0 = sm + (2 * i) * kColsA + c;
-            u64 a0 = p0[0], a1 = p0[kColsA];
-            ct_bfly(a0, a1, stw[(1 << s) + i], q, q2);
-            p0[0] = a0;
-            p0[kColsA] = a1;
-        }
-        __syncthreads();
-    }
-    for (int idx = threadIdx.x; idx < N1 * kColsA; idx += kNttThreads)
-        dst[(size_t)(idx >> LC) * N2 + c0 + (idx & (kColsA - 1))] = sm[idx];   // lazy, < 4q
-}
-
-template <int LOGN>
-__global__ void __launch_bounds__(kNttThreads)
-ntt_fwd_b(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ tw)
-{
-    constexpr int S1 = LOGN / 2, N = 1 << LOGN, N1 = 1 << S1, LN2 = LOGN - S1, N2 = 1 << LN2;
-    constexpr int R = (kElemsB / N2) < N1 ? (kElemsB / N2) : N1;
-    const int limb = blockIdx.y;
-    const int col = limb % bt.per_row, row = limb / bt.per_row;
-    const int pi = bt.pidx[col];
-    if (pi < 0) return;
-    extern __shared__ u64 sm[];
-    const u64 q = primes[pi].q, q2 = 2 * q;
-    const ulonglong2 *twp = tw + (size_t)pi * N;
-    const int row0 = blockIdx.x * R;
-    u64 *d = bt.dst + ((size_t)row * bt.dst_stride + col) * N + (size_t)row0 * N2;
-    for (int idx = threadIdx.x; idx < R * N2; idx += kNttThreads) sm[idx] = d[idx];
-    __syncthreads();
-    int ls = 0;   // stage inside the row; global stage S1 + ls
-#pragma unroll
-    for (; ls + 1 < LN2; ls += 2) {
-        const int s = S1 + ls;
-        const int lq = LN2 - ls - 2;
-#pragma unroll 2
-        for (int b = threadIdx.x; b < R * (N2 / 4); b += kNttThreads) {
-            const int r = b >> (LN2 - 2), u = b & (N2 / 4 - 1);
-            const int i = u >> lq, j = u & ((1 << lq) - 1);
-            const int pos = (i << (lq + 2)) + j;
-            const int gi = ((row0 + r) << ls) + i;
-            const ulonglong2 w1 = twp[(1 << s) + gi];
-            const ulonglong2 w2 = twp[(2 << s) + 2 * gi], w3 = twp[(2 << s) + 2 * gi + 1];
-            u64 *p0 = sm + r * N2 + pos;
-            const int dq = 1 << lq;
-            u64 a0 = p0[0], a1 = p0[dq], a2 = p0[2 * dq], a3 = p0[3 * dq];
-            ct_bfly(a0, a2, w1, q, q2);
-            ct_bfly(a1, a3, w1, q, q2);
-            ct_bfly(a0, a1, w2, q, q2);
-            ct_bfly(a2, a3, w3, q, q2);
-            p0[0] = a0;
-            p0[dq] = a1;
-            p0[2 * dq] = a2;
-            p0[3 * dq] = a3;
-        }
-        __syncthreads();
-    }
-    if (ls < LN2) {   // last radix-2 stage, half distance 1
-        const int s = S1 + ls;
-        for (int b = threadIdx.x; b < R * (N2 / 2); b += kNttThreads) {
-            const int r = b >> (LN2 - 1), i = b & (N2 / 2 - 1);
-            u64 *p0 = sm + r * N2 + 2 * i;
-            u64 a0 = p0[0], a1 = p0[1];
-            ct_bfly(a0, a1, twp[(1 << s) + ((row0 + r) << ls) + i], q, q2);
-            p0[0] = a0;
-            p0[1] = a1;
-        }
-        __syncthreads();
-    }
-    for (int idx = threadIdx.x; idx < R * N2; idx += kNttThreads) d[idx] = reduce4(sm[idx], q);
-}
-
-template <int LOGN>
-__global__ void __launch_bounds__(kNttThreads)
-ntt_inv_b(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ itw)
-{
-    constexpr int S1 = LOGN / 2, N = 1 << LOGN, N1 = 1 << S1, LN2 = LOGN - S1, N2 = 1 << LN2;
-    constexpr int R = (kElemsB / N2) < N1 ? (kElemsB / N2) : N1;
-    const int limb = blockIdx.y;
-    const int col = limb % bt.per_row, row = limb / bt.per_row;
-    const int pi = bt.pidx[col];
-    if (pi < 0) return;
-    extern __shared__ u64 sm[];
-    const u64 q = primes[pi].q, q2 = 2 * q;
-    const ulonglong2 *twp = itw + (size_t)pi * N;
-    const int row0 = blockIdx.x * R;
-    const u64 *sr = bt.src + ((size_t)row * bt.src_stride + col) * N + (size_t)row0 * N2;
-    u64 *d = bt.dst + ((size_t)row * bt.dst_stride + col) * N + (size_t)row0 * N2;
-    for (int idx = threadIdx.x; idx < R * N2; idx += kNttThreads) sm[idx] = sr[idx];
-    __syncthreads();
-    int ls = LN2 - 1;
-    if (LN2 & 1) {   // odd: the last stage (half distance 1) alone first
-        const int s = S1 + ls;
-        for (int b = threadIdx.x; b < R * (N2 / 2); b += kNttThreads) {
-            const int r = b >> (LN2 - 1), i = b & (N2 / 2 - 1);
-            u64 *p0 = sm + r * N2 + 2 * i;
-            u64 a0 = p0[0], a1 = p0[1];
-            gs_bfly(a0, a1, twp[(1 << s) + ((row0 + r) << ls) + i], q, q2);
-            p0[0] = a0;
-            p0[1] = a1;
-        }
-        __syncthreads();
-        ls--;
-    }
-#pragma unroll
-    for (; ls >= 1; ls -= 2) {   // stages (ls-1, ls), higher one first
-        const int lo = ls - 1, s = S1 + lo;
-        const int lq = LN2 - lo - 2;
-#pragma unroll 2
-        for (int b = threadIdx.x; b < R * (N2 / 4); b += kNttThreads) {
-            const int r = b >> (LN2 - 2), u = b & (N2 / 4 - 1);
-            const int i = u >> lq, j = u & ((1 << lq) - 1);
-            const int pos = (i << (lq + 2)) + j;
-            const int gi = ((row0 + r) << lo) + i;
-            const ulonglong2 w1 = twp[(1 << s) + gi];
-            const ulonglong2 w2 = twp[(2 << s) + 2 * gi], w3 = twp[(2 << s) + 2 * gi + 1];
-            u64 *p0 = sm + r * N2 + pos;
-            const int dq = 1 << lq;
-            u64 a0 = p0[0], a1 = p0[dq], a2 = p0[2 * dq], a3 = p0[3 * dq];
-            gs_bfly(a0, a1, w2, q, q2);
-            gs_bfly(a2, a3, w3, q, q2);
-            gs_bfly(a0, a2, w1, q, q2);
-            gs_bfly(a1, a3, w1, q, q2);
-            p0[0] = a0;
-            p0[dq] = a1;
-            p0[2 * dq] = a2;
-            p0[3 * dq] = a3;
-        }
-        __syncthreads();
-    }
-    for (int idx = threadIdx.x; idx < R * N2; idx += kNttThreads) d[idx] = sm[idx];   // < 2q
-}
-
-template <int LOGN>
-__global__ void __launch_bounds__(kNttThreads)
-ntt_inv_a(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ itw,
-          const u64 *__restrict__ ninv)
-{
-    constexpr int S1 = LOGN / 2, N = 1 << LOGN, N1 = 1 << S1, N2 = N >> S1;
-    constexpr int LC = 4;
-    const int limb = blockIdx.y;
-    const int col = limb % bt.per_row, row = limb / bt.per_row;
-    const int pi = bt.pidx[col];
-    if (pi < 0) return;
-    extern __shared__ u64 sm[];
-    ulonglong2 *stw = reinterpret_cast<ulonglong2 *>(sm + N1 * kColsA);
-    const u64 q = primes[pi].q, q2 = 2 * q;
-    const ulonglong2 *twp = itw + (size_t)pi * N;
-    u64 *d = bt.dst + ((size_t)row * bt.dst_stride + col) * N;
-    const int c0 = blockIdx.x * kColsA;
-    for (int i = threadIdx.x; i < N1; i += kNttThreads) stw[i] = twp[i];
-    for (int idx = threadIdx.x; idx < N1 * kColsA; idx += kNttThreads)
-        sm[idx] = d[(size_t)(idx >> LC) * N2 + c0 + (idx & (kColsA - 1))];
-    __syncthreads();
-    int s = S1 - 1;
-    if (S1 & 1) {   // odd: last stage (h = 1) alone first
-        for (int b = threadIdx.x; b < (N1 / 2) * kColsA; b += kNttThreads) {
-            const int c = b & (kColsA - 1), i = b >> LC;
-            u64 *p0 = sm + (2 * i) * kColsA + c;
-            u64 a0 = p0[0], a1 = p0[kColsA];
-            gs_bfly(a0, a1, stw[(1 << s) + i], q, q2);
-            p0[0] = a0;
-            p0[kColsA] = a1;
-        }
-        __syncthreads();
-        s--;
-    }
-#pragma unroll
-    for (; s >= 1; s -= 2) {   // stages (s-1, s), higher one first
-        const int lo = s - 1;
-        const int lq = S1 - lo - 2;
-#pragma unroll 2
-        for (int b = threadIdx.x; b < (N1 / 4) * kColsA; b += kNttThreads) {
-            const int c = b & (kColsA - 1), u = b >> LC;
-            const int i = u >> lq, j = u & ((1 << lq) - 1);
-            const int r = (i << (lq + 2)) + j;
-            const ulonglong2 w1 = stw[(1 << lo) + i];
-            const ulonglong2 w2 = stw[(2 << lo) + 2 * i], w3 = stw[(2 << lo) + 2 * i + 1];
-            u64 *p0 = sm + r * kColsA + c;
-            const int dq = (1 << lq) * kColsA;
-            u64 a0 = p0[0], a1 = p0[dq], a2 = p0[2 * dq], a3 = p0[3 * dq];
-            gs_bfly(a0, a1, w2, q, q2);
-            gs_bfly(a2, a3, w3, q, q2);
-            gs_bfly(a0, a2, w1, q, q2);
-            gs_bfly(a1, a3, w1, q, q2);
-            p0[0] = a0;
-            p0[dq] = a1;
-            p0[2 * dq] = a2;
-            p0[3 * dq] = a3;
-        }
-        __syncthreads();
-    }
-    const u64 ni = ninv[2 * pi], nis = ninv[2 * pi + 1];
-    for (int idx = threadIdx.x; idx < N1 * kColsA; idx += kNttThreads)
-        d[(size_t)(idx >> LC) * N2 + c0 + (idx & (kColsA - 1))] = shoup_mul(sm[idx], ni, nis, q);
 }
 
 // ------------------------------------------------------------------------
@@ -1361,28 +1015,6 @@ static void ntt16_pass_b_od(fg_ctx *ctx, const Batch &bt, int count)
         ntt16_fwd_b<16, OD><<<dim3(16, count), 256, 0, ctx->stream>>>(bt, ctx->d_primes, fwd, rows);
 }
 
-template <int LOGN>
-static void ntt_launch_t(fg_ctx *ctx, const Batch &bt, int count, bool inverse)
-{
-    constexpr int S1 = LOGN / 2, N = 1 << LOGN, N1 = 1 << S1, N2 = N >> S1;
-    constexpr int R = (kElemsB / N2) < N1 ? (kElemsB / N2) : N1;
-    const size_t smA = (size_t)N1 * kColsA * 8 + (size_t)N1 * 16;
-    const size_t smB = (size_t)R * N2 * 8;
-    const auto *fwd = (const ulonglong2 *)ctx->d_fwd;
-    const auto *inv = (const ulonglong2 *)ctx->d_inv;
-    dim3 gA(N2 / kColsA, count), gB(N1 / R, count);
-    Batch b2 = bt;
-    b2.src = b2.dst;
-    b2.src_stride = b2.dst_stride;
-    if (!inverse) {
-        ntt_fwd_a<LOGN><<<gA, kNttThreads, smA, ctx->stream>>>(bt, ctx->d_primes, fwd);
-        ntt_fwd_b<LOGN><<<gB, kNttThreads, smB, ctx->stream>>>(b2, ctx->d_primes, fwd);
-    } else {
-        ntt_inv_b<LOGN><<<gB, kNttThreads, smB, ctx->stream>>>(bt, ctx->d_primes, inv);
-        ntt_inv_a<LOGN><<<gA, kNttThreads, smA, ctx->stream>>>(b2, ctx->d_primes, inv, ctx->d_ninv);
-    }
-}
-
 static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool inverse)
 {
     FG_CHECK(src.per_row == dst.per_row && src.rows == dst.rows, FG_EINVAL, "ntt: shape mismatch");
@@ -1394,16 +1026,11 @@ static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool
     int active = 0;
     for (int v : src.pidx) active += v >= 0;
     KTimer kt(ctx, "ntt", (double)active * src.rows * ctx->n * 8 * 2);
-    switch (ctx->log_n) {
-    case 10: ntt_launch_t<10>(ctx, bt, count, inverse); break;
-    case 11: ntt_launch_t<11>(ctx, bt, count, inverse); break;
-    case 12: ntt_launch_t<12>(ctx, bt, count, inverse); break;
-    case 13: ntt_launch_t<13>(ctx, bt, count, inverse); break;
-    case 14: ntt_launch_t<14>(ctx, bt, count, inverse); break;
-    case 15: ntt_launch_t<15>(ctx, bt, count, inverse); break;
-    case 16: ntt16_launch(ctx, bt, count, inverse); break;
-    default: throw fg_error(FG_EINVAL, "ntt: unsupported ring degree");
+    if (ctx->log_n < 16) {
+        ntt_small(ctx, bt, count, inverse);
+        return;
     }
+    ntt16_launch(ctx, bt, count, inverse);
     check_launch("ntt", 2);
 }
 
