@@ -83,15 +83,15 @@ __device__ __forceinline__ void fwd_a16_rounds(u64 (&v)[16], u64 *d, const ulong
 {
     const int t = threadIdx.x, c = t % COLS, r = t / COLS;   // r: r0 in round 1, r1 in round 2
     constexpr int N2 = 256;
-    const u64 q2 = 2 * q;
+    const u64 q4 = 4 * q;
     // stage st, group g at (1 << st) + g
-    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q4);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[(r + 16 * m) * COLS + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[(16 * r + m) * COLS + c];
-    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q4);
 #pragma unroll
     for (int m = 0; m < 16; m++) d[(size_t)(16 * r + m) * N2 + c] = v[m];   // lazy
 }
@@ -134,13 +134,13 @@ __device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, cons
 {
     const int t = threadIdx.x, j = t & 15, r = t >> 4;
     constexpr int S1 = 8;
-    const u64 q = P.q, q2 = 2 * q;
+    const u64 q = P.q, q4 = 4 * q;
     u64 v[16];
     const int grow = row0 + r;
     u64 *drow = d + (size_t)r * 256;
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = drow[j + 16 * m];
-    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2);
+    ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q4);
     u64 *srow = sm + r * kR16Row;
 #pragma unroll
     for (int m = 0; m < 16; m++) srow[pad16(j + 16 * m)] = v[m];
@@ -149,12 +149,12 @@ __device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, cons
     for (int m = 0; m < 16; m++) v[m] = srow[pad16(16 * j + m)];
     // row stages 12..15 from the row-blocked table (consecutive per row)
     ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
-               q, q2);
+               q, q4);
     ulonglong2 *o = reinterpret_cast<ulonglong2 *>(drow + 16 * j);
 #pragma unroll
     for (int m = 0; m < 16; m += 2)
         o[m / 2] = LAZY ? make_ulonglong2(reduce_word(v[m], P), reduce_word(v[m + 1], P))
-                        : make_ulonglong2(reduce4(v[m], q), reduce4(v[m + 1], q));
+                        : make_ulonglong2(reduce8(v[m], q), reduce8(v[m + 1], q));
 }
 
 template <int ROWS, bool OD>
@@ -182,7 +182,7 @@ __device__ __forceinline__ void inv_b16_body(const u64 *s, u64 *d, const ulonglo
 {
     const int t = threadIdx.x, j = t & 15, r = t >> 4;
     constexpr int S1 = 8;
-    const u64 q2 = 2 * q;
+    const u64 q4 = 4 * q;
     u64 v[16];
     const int grow = row0 + r;
     const ulonglong2 *in = reinterpret_cast<const ulonglong2 *>(s + (size_t)r * 256 + 16 * j);
@@ -193,17 +193,17 @@ __device__ __forceinline__ void inv_b16_body(const u64 *s, u64 *d, const ulonglo
         v[m + 1] = a.y;
     }
     gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
-               q, q2, 0);
+               q, q4, 0);
     u64 *srow = sm + r * kR16Row;
 #pragma unroll
     for (int m = 0; m < 16; m++) srow[pad16(16 * j + m)] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = srow[pad16(j + 16 * m)];
-    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q2, 4);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return twp[(1 << (S1 + st)) + (grow << st) + g]; }), q, q4, 4);
     u64 *drow = d + (size_t)r * 256;
 #pragma unroll
-    for (int m = 0; m < 16; m++) drow[j + 16 * m] = v[m];   // lazy (< 2^9 q or < 2q)
+    for (int m = 0; m < 16; m++) drow[j + 16 * m] = v[m];   // lazy (< 2^9 q or < 4q)
 }
 
 template <int ROWS, bool OD>
@@ -232,17 +232,17 @@ __device__ __forceinline__ void inv_a16_body(u64 *d, const ulonglong2 *stw, u64 
 {
     const int t = threadIdx.x, c = t % COLS, r = t / COLS;
     constexpr int N2 = 256;
-    const u64 q2 = 2 * q;
+    const u64 q4 = 4 * q;
     u64 v[16];
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = d[(size_t)(16 * r + m) * N2 + c];
-    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q2, 8);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << (st + 4)) + (r << st) + g]; }), q, q4, 8);
 #pragma unroll
     for (int m = 0; m < 16; m++) sm[(16 * r + m) * COLS + c] = v[m];
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = sm[(r + 16 * m) * COLS + c];
-    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q2, 12);
+    gs_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return stw[(1 << st) + g]; }), q, q4, 12);
 #pragma unroll
     for (int m = 0; m < 16; m++) d[(size_t)(r + 16 * m) * N2 + c] = shoup_mul(v[m], ni, nis, q);
 }

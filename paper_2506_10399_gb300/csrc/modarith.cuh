@@ -1,6 +1,6 @@
 // modarith.cuh -- 64-bit modular arithmetic on CUDA cores for RNS-CKKS.
 //
-// All primes are below 2^62, so lazy values in [0, 4q) fit a 64-bit word.
+// All primes are below 2^60, so lazy values in [0, 8q) fit a 64-bit word.
 // Methods (each a published one):
 //   * Shoup's precomputed-quotient multiplication by a fixed operand w
 //     (w' = floor(w 2^64 / q)), lazy form in [0, 2q) as in Harvey, "Faster
@@ -31,8 +31,10 @@ __device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q)
 
 __device__ __forceinline__ u64 reduce2(u64 x, u64 q) { return x >= q ? x - q : x; }
 
-__device__ __forceinline__ u64 reduce4(u64 x, u64 q)
+// x below 8q
+__device__ __forceinline__ u64 reduce8(u64 x, u64 q)
 {
+    x = x >= 4 * q ? x - 4 * q : x;
     x = x >= 2 * q ? x - 2 * q : x;
     return x >= q ? x - q : x;
 }

@@ -82,9 +82,9 @@ __device__ __forceinline__ void fwd_round(u64 (&v)[16], int t, const Tw<LS, S0> 
         if (last && K == Rounds<LS>::n - 1) {
             const ulonglong2 *p = last + A::T * g;
             ct_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return __ldg(p + (size_t)((1 << st) - 1 + x) * nb); },
-                                 q, 2 * q);
+                                 q, 4 * q);
         } else {
-            ct_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return tw(A::s, st, blk, x); }, q, 2 * q);
+            ct_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return tw(A::s, st, blk, x); }, q, 4 * q);
         }
     }
 }
@@ -100,9 +100,9 @@ __device__ __forceinline__ void inv_round(u64 (&v)[16], int t, const Tw<LS, S0> 
         if (last && K == Rounds<LS>::n - 1) {
             const ulonglong2 *p = last + A::T * g;
             gs_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return __ldg(p + (size_t)((1 << st) - 1 + x) * nb); },
-                                 q, 2 * q, k0);
+                                 q, 4 * q, k0);
         } else {
-            gs_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return tw(A::s, st, blk, x); }, q, 2 * q, k0);
+            gs_round<A::R, LAZY>(v + g * A::R, [&](int st, int x) { return tw(A::s, st, blk, x); }, q, 4 * q, k0);
         }
     }
 }
@@ -224,7 +224,7 @@ ntt_rows_fwd(const __grid_constant__ Batch bt, const PrimeC *__restrict__ primes
     } else {
         fwd_all<LS, W::S0, false>(v, t, s, W::pad(), w, last, W::NB, P.q);
 #pragma unroll
-        for (int m = 0; m < 16; m++) v[m] = reduce4(v[m], P.q);
+        for (int m = 0; m < 16; m++) v[m] = reduce8(v[m], P.q);
     }
     W::store(v, dst, t);
 }
@@ -252,7 +252,7 @@ ntt_rows_inv(const __grid_constant__ Batch bt, const PrimeC *__restrict__ primes
     u64 *dst = bt.dst + ((size_t)lrow * bt.dst_stride + col) * N + ((size_t)row << LS);
     const u64 ni = ninv[2 * pi], nis = ninv[2 * pi + 1];
 #pragma unroll
-    for (int m = 0; m < 16; m++)   // whole limbs: scaled; else lazy (< 2^(LS + 1) q or < 2q)
+    for (int m = 0; m < 16; m++)   // whole limbs: scaled; else lazy (< 2^(LS + 1) q or < 4q)
         dst[A::elem(t, m / A::R, m % A::R)] = LS == LOGN ? shoup_mul(v[m], ni, nis, q) : v[m];
 }
 
