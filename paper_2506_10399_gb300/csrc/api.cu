@@ -1169,8 +1169,10 @@ int fg_poly_mul(fg_ctx *ctx, const uint64_t *a, const uint64_t *b, int level, ui
     kern::ntt_fwd(ctx, sa, ta_s);
     kern::ntt_fwd(ctx, sb, tb_s);
     kern::pointwise(ctx, ta, tb, ta, nl, pid);
-    kern::ntt_inv(ctx, ta_s, ta_s);
-    stage_out(ctx, c, ta, (size_t)nl * N);
+    u64 *o = is_device_ptr(c) ? c : ta;   // the operands have been read
+    kern::LimbSet os{o, nl, nl, 1, pid};
+    kern::ntt_inv(ctx, ta_s, os);
+    stage_out(ctx, c, o, (size_t)nl * N);
     sync(ctx);
     API_CATCH(ctx)
 }
@@ -1228,40 +1230,24 @@ int fg_mul_relin_rescale(fg_ctx *ctx, const fg_keys *keys, const uint64_t *a, co
         kern::LimbSet bs{const_cast<u64 *>(db), nl, nl, 2 * n, pid}, bn{B, nl, nl, 2 * n, pid};
         kern::ntt_fwd(ctx, bs, bn);
     }
-    // lane (d0, d2) per pair, d1 aside (NTT domain)
+    // lane (d0, d2) per pair, P d1 aside (NTT domain)
     u64 *Ln = (u64 *)ctx->buf("mul_lane", w * 8);
     u64 *D1 = (u64 *)ctx->buf("mul_d1", (size_t)n * pw * 8);
-    u64 *T = (u64 *)ctx->buf("mul_t", (size_t)n * pw * 8);
-    for (int c = 0; c < n; c++) {
-        const u64 *a0 = A + (size_t)c * 2 * pw, *a1 = a0 + pw;
-        const u64 *b0 = B + (size_t)c * 2 * pw, *b1 = b0 + pw;
-        u64 *l0 = Ln + (size_t)c * 2 * pw;
-        kern::pointwise(ctx, a0, b0, l0, nl, pid);
-        kern::pointwise(ctx, a1, b1, l0 + pw, nl, pid);
-        kern::pointwise(ctx, a0, b1, D1 + (size_t)c * pw, nl, pid);
-        kern::pointwise(ctx, a1, b0, T + (size_t)c * pw, nl, pid);
-    }
-    kern::add(ctx, D1, T, D1, n * nl, pid);
+    kern::tensor(ctx, A, B, Ln, D1, n, nl);
     // u = KS(d2) + P d0 (part 0), then + P d1 (part 1): ModDown gives
     // (d0, d1) + KS(d2) exactly, and the rescale is fused into it
     u64 *digits = (u64 *)ctx->buf("mul_digits", (size_t)n * beta * E * N * 8);
     kern::modup(ctx, Ln, nl, n, level, digits);
     u64 *u = (u64 *)ctx->buf("mul_u", (size_t)n * 2 * E * N * 8);
     kern::ks_multi(ctx, {&rk}, {u}, Ln, nl, n, level, digits);
-    kern::scalar(ctx, D1, T, n * nl, pid, ctx->d_pmodq);
-    for (int c = 0; c < n; c++) {
-        u64 *u1 = u + ((size_t)c * 2 + 1) * E * N;
-        kern::add(ctx, u1, T + (size_t)c * pw, u1, nl, pid);
-    }
+    kern::add_part1(ctx, u, E, D1, n, nl);
     u64 *R = (u64 *)ctx->buf("mul_r", w * 8);
     kern::moddown_rescale_to_lane(ctx, u, n, level, R, nl);
-    std::vector<int> top(nl, -1);
-    for (int i = 0; i < level; i++) top[i] = i;
-    kern::LimbSet rs{R, nl, nl, 2 * n, top};
-    kern::ntt_inv(ctx, rs, rs);
     const size_t ow = (size_t)n * 2 * level * N;
     u64 *O = is_device_ptr(out) ? out : (u64 *)ctx->buf("mul_o", ow * 8);
-    kern::copy_limbs(ctx, R, nl, O, level, 2 * n, level);
+    const std::vector<int> kept = iota(level);
+    kern::LimbSet rs{R, nl, level, 2 * n, kept}, os{O, level, level, 2 * n, kept};
+    kern::ntt_inv(ctx, rs, os);
     if (O != out) stage_out(ctx, out, O, ow);
     sync(ctx);
     API_CATCH(ctx)
@@ -1290,9 +1276,10 @@ int fg_rotate(fg_ctx *ctx, const fg_keys *keys, const uint64_t *ct, int level, i
                                   (size_t)ctx->n_digits(level) * ctx->ext(level) * N * 8);
     kern::modup(ctx, lane, nl, 1, level, digits);
     kern::rotate(ctx, key, lane, nl, 1, level, digits, res, nl);
-    kern::LimbSet rs{res, nl, nl, 2, pid};
-    kern::ntt_inv(ctx, rs, rs);
-    stage_out(ctx, out, res, (size_t)2 * nl * N);
+    u64 *o = is_device_ptr(out) ? out : res;   // the input has been read
+    kern::LimbSet rs{res, nl, nl, 2, pid}, os{o, nl, nl, 2, pid};
+    kern::ntt_inv(ctx, rs, os);
+    stage_out(ctx, out, o, (size_t)2 * nl * N);
     sync(ctx);
     API_CATCH(ctx)
 }

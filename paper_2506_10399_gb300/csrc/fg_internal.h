@@ -313,6 +313,10 @@ void from_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx);
 void pointwise(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count,
                const std::vector<int> &pidx);
 void add(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count, const std::vector<int> &pidx);
+// tensor product of n pairs [n][2][nl][N]: lane = (a0 b0, a1 b1), d1 = P (a0 b1 + a1 b0) [n][nl][N]
+void tensor(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *lane, u64 *d1, int n, int nl);
+// part 1 of u [n][2][E][N] += d [n][nl][N]
+void add_part1(fg_ctx *ctx, u64 *u, int E, const u64 *d, int n, int nl);
 void neg(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &pidx);
 // c = a * s[c % period] with d_scal = (w, w') pairs per limb column
 void scalar(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &pidx,
@@ -374,8 +378,8 @@ void ks_launch(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::
 void ks_multi(fg_ctx *ctx, const std::vector<const KeyDev *> &keys, const std::vector<u64 *> &us,
               const u64 *lane, int ls, int ncol, int level, const u64 *digits);
 // ModDown of an extended-basis sum to Q, then the rescale by q_level, into a
-// lane (limbs 0..level-1); ext is scratch and is overwritten
-void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls);
+// lane (limbs 0..level-1), or added to it; ext is scratch and is overwritten
+void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls, bool accumulate = false);
 // residues mod the special primes from limb 0 (centred): out [np][N]
 void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out);
 // every destination gets mask (x) lane

@@ -128,9 +128,9 @@ ntt16_fwd_a(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 
     else fwd_a16_body<false, COLS, OD>(src, dst, stw, q, sm);
 }
 
-template <bool LAZY, bool OD>
-__device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, const ulonglong2 *rows,
-                                             int row0, const PrimeC &P, u64 *sm)
+template <bool LAZY, bool OD, bool FIN>
+__device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, const ulonglong2 *rows, int row0,
+                                             const PrimeC &P, u64 *sm, const Finish &fin, int lrow, int lcol)
 {
     const int t = threadIdx.x, j = t & 15, r = t >> 4;
     constexpr int S1 = 8;
@@ -150,17 +150,16 @@ __device__ __forceinline__ void fwd_b16_body(u64 *d, const ulonglong2 *twp, cons
     // row stages 12..15 from the row-blocked table (consecutive per row)
     ct_round<16, LAZY>(v, twiddles<OD>([&](int st, int g) { return rows[((size_t)grow * 15 + (1 << st) - 1 + g) * 16 + j]; }),
                q, q4);
-    ulonglong2 *o = reinterpret_cast<ulonglong2 *>(drow + 16 * j);
+    // d: the tile's first word, row0 rows into the limb
 #pragma unroll
     for (int m = 0; m < 16; m += 2)
-        o[m / 2] = LAZY ? make_ulonglong2(reduce_word(v[m], P), reduce_word(v[m + 1], P))
-                        : make_ulonglong2(reduce8(v[m], q), reduce8(v[m + 1], q));
+        put_pair<LAZY, FIN>(v[m], v[m + 1], d - (size_t)row0 * 256, (size_t)grow * 256 + 16 * j + m, fin, lrow, lcol, 65536, P);
 }
 
-template <int ROWS, bool OD>
+template <int ROWS, bool OD, bool FIN>
 __global__ void __launch_bounds__(16 * ROWS, (OD ? 64 : 48) / ROWS)
 ntt16_fwd_b(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ tw,
-            const ulonglong2 *__restrict__ tw_rows)
+            const ulonglong2 *__restrict__ tw_rows, const Finish fin)
 {
     const int limb = blockIdx.y;
     const int col = limb % bt.per_row, row = limb / bt.per_row;
@@ -172,8 +171,8 @@ ntt16_fwd_b(const Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 
     const int row0 = blockIdx.x * ROWS;
     u64 *d = bt.dst + ((size_t)row * bt.dst_stride + col) * 65536 + (size_t)row0 * 256;
     const ulonglong2 *rows = tw_rows + (size_t)pi * 256 * 15 * 16;
-    if (P.q < (1ull << 47)) fwd_b16_body<true, OD>(d, twp, rows, row0, P, sm);
-    else fwd_b16_body<false, OD>(d, twp, rows, row0, P, sm);
+    if (P.q < (1ull << 47)) fwd_b16_body<true, OD, FIN>(d, twp, rows, row0, P, sm, fin, row, col);
+    else fwd_b16_body<false, OD, FIN>(d, twp, rows, row0, P, sm, fin, row, col);
 }
 
 template <bool LAZY, bool OD>
@@ -367,6 +366,34 @@ __global__ void k_pointwise(const u64 *a, const u64 *b, u64 *c, const Batch bt,
     const size_t off = (size_t)limb * N;
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N; x += gridDim.x * blockDim.x)
         c[off + x] = mont_mul(mont_mul(a[off + x], b[off + x], P), P.r2, P);
+}
+
+// Tensor product of n pairs (a0, a1) x (b0, b1) (NTT domain, [n][2][nl][N]):
+// lane = (a0 b0, a1 b1), d1 = P (a0 b1 + a1 b0), one pass over the operands
+// instead of four products, a sum and a scaling each through memory.
+__global__ void __launch_bounds__(256)
+k_tensor(const u64 *a, const u64 *b, u64 *lane, u64 *d1, int nl, const PrimeC *__restrict__ primes,
+         const u64 *__restrict__ pmodq, int N)
+{
+    const int i = blockIdx.y, c = blockIdx.z, x = blockIdx.x * blockDim.x + threadIdx.x;
+    const PrimeC P = primes[i];
+    const u64 pr2 = mont_mul(mont_mul(pmodq[2 * i], P.r2, P), P.r2, P);   // P R^2
+    const size_t o0 = ((size_t)c * 2 * nl + i) * N + x, o1 = o0 + (size_t)nl * N;
+    const u64 a0 = a[o0], a1 = a[o1], b0 = b[o0], b1 = b[o1];
+    lane[o0] = mont_mul(mont_mul(a0, b0, P), P.r2, P);
+    lane[o1] = mont_mul(mont_mul(a1, b1, P), P.r2, P);
+    u64 hi = mulhi64(a0, b1), lo = a0 * b1;   // the sum of two products is below q 2^64
+    mac128(hi, lo, a1, b0);
+    d1[((size_t)c * nl + i) * N + x] = mont_mul(redc(hi, lo, P), pr2, P);
+}
+
+// part 1 of n extended ciphertexts u [n][2][E][N] += d [n][nl][N] on the limbs of Q
+__global__ void __launch_bounds__(256)
+k_add_part1(u64 *u, int E, const u64 *__restrict__ d, int nl, const PrimeC *__restrict__ primes, int N)
+{
+    const int i = blockIdx.y, c = blockIdx.z, x = blockIdx.x * blockDim.x + threadIdx.x;
+    u64 *p = u + (((size_t)c * 2 + 1) * E + i) * N + x;
+    *p = add_mod(*p, d[((size_t)c * nl + i) * N + x], primes[i].q);
 }
 
 __global__ void k_add(const u64 *a, const u64 *b, u64 *c, const Batch bt,
@@ -810,25 +837,6 @@ k_moddown_rescale_conv(const u64 *__restrict__ ext, int E, u64 *w, int l,
     }
 }
 
-// out_i = (ext_i - w_i) (P q_l)^-1 for i < l (NTT domain)
-__global__ void __launch_bounds__(256)
-k_moddown_rescale_finish(const u64 *__restrict__ ext, int E, const u64 *__restrict__ w, u64 *out,
-                         int ls, int npoly, int l, const u64 *__restrict__ tab,
-                         const PrimeC *__restrict__ primes, int N)
-{
-    const int i = blockIdx.y;
-    const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (x >= N) return;
-    const u64 q = primes[i].q, c = tab[2 * i], cs = tab[2 * i + 1];
-    for (int poly = 0; poly < npoly; poly++) {
-        const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(ext + ((size_t)poly * E + i) * N + x);
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(w + ((size_t)poly * l + i) * N + x);
-        *reinterpret_cast<ulonglong2 *>(out + ((size_t)poly * ls + i) * N + x) =
-            make_ulonglong2(shoup_mul(sub_mod(e.x, v.x, q), c, cs, q),
-                            shoup_mul(sub_mod(e.y, v.y, q), c, cs, q));
-    }
-}
-
 // ModDown + rescale at N = 2^16, the conversion fused into the first NTT
 // pass of w (see k_moddown_rescale_conv for what w is).  First
 // k_moddown_prep, per coefficient of each polynomial: y_k (the inverse NTT
@@ -964,8 +972,22 @@ KTimer::~KTimer()
 }
 
 
+// N = 2^16 forward pass B alone (the whole second half of a transform), in
+// place on bt.dst or finished
+template <bool OD>
+static void ntt16_pass_b_od(fg_ctx *ctx, const Batch &bt, int count, const Finish *fin = nullptr)
+{
+    const auto *fwd = (const ulonglong2 *)ctx->d_fwd;
+    const auto *rows = (const ulonglong2 *)ctx->d_fwd_rows;
+    const int R = ctx->tune.ntt_rows == 8 ? 8 : 16;
+    auto kern = R == 8 ? (fin ? ntt16_fwd_b<8, OD, true> : ntt16_fwd_b<8, OD, false>)
+                       : (fin ? ntt16_fwd_b<16, OD, true> : ntt16_fwd_b<16, OD, false>);
+    kern<<<dim3(256 / R, count), 16 * R, 0, ctx->stream>>>(bt, ctx->d_primes, fwd, rows, fin ? *fin : Finish());
+}
+
 template <int COLS, int ROWS, bool OD>
-static void ntt16_launch_t(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const u64 *col_scale)
+static void ntt16_launch_t(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const u64 *col_scale,
+                           const Finish *fin)
 {
     const auto *fwd = (const ulonglong2 *)ctx->d_fwd;
     const auto *inv = (const ulonglong2 *)ctx->d_inv;
@@ -975,8 +997,7 @@ static void ntt16_launch_t(fg_ctx *ctx, const Batch &bt, int count, bool inverse
     b2.src_stride = b2.dst_stride;
     if (!inverse) {
         ntt16_fwd_a<COLS, OD><<<gA, 16 * COLS, 0, ctx->stream>>>(bt, ctx->d_primes, fwd);
-        ntt16_fwd_b<ROWS, OD><<<gB, 16 * ROWS, 0, ctx->stream>>>(b2, ctx->d_primes, fwd,
-                                                                (const ulonglong2 *)ctx->d_fwd_rows);
+        ntt16_pass_b_od<OD>(ctx, b2, count, fin);
     } else {
         ntt16_inv_b<ROWS, OD><<<gB, 16 * ROWS, 0, ctx->stream>>>(bt, ctx->d_primes, inv,
                                                                 (const ulonglong2 *)ctx->d_inv_rows);
@@ -987,35 +1008,24 @@ static void ntt16_launch_t(fg_ctx *ctx, const Batch &bt, int count, bool inverse
 
 // the tile and twiddle form of the N = 2^16 transform from the context's tuning
 template <bool OD>
-static void ntt16_launch_od(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const u64 *col_scale)
+static void ntt16_launch_od(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const u64 *col_scale,
+                            const Finish *fin)
 {
     const bool ca = ctx->tune.ntt_cols == 8, rb = ctx->tune.ntt_rows == 8;
-    if (!ca && !rb) ntt16_launch_t<16, 16, OD>(ctx, bt, count, inverse, col_scale);
-    else if (ca && !rb) ntt16_launch_t<8, 16, OD>(ctx, bt, count, inverse, col_scale);
-    else if (!ca && rb) ntt16_launch_t<16, 8, OD>(ctx, bt, count, inverse, col_scale);
-    else ntt16_launch_t<8, 8, OD>(ctx, bt, count, inverse, col_scale);
+    if (!ca && !rb) ntt16_launch_t<16, 16, OD>(ctx, bt, count, inverse, col_scale, fin);
+    else if (ca && !rb) ntt16_launch_t<8, 16, OD>(ctx, bt, count, inverse, col_scale, fin);
+    else if (!ca && rb) ntt16_launch_t<16, 8, OD>(ctx, bt, count, inverse, col_scale, fin);
+    else ntt16_launch_t<8, 8, OD>(ctx, bt, count, inverse, col_scale, fin);
 }
 
 static void ntt16_launch(fg_ctx *ctx, const Batch &bt, int count, bool inverse,
-                         const u64 *col_scale = nullptr)
+                         const u64 *col_scale = nullptr, const Finish *fin = nullptr)
 {
-    if (ctx->tune.ntt_tw) ntt16_launch_od<true>(ctx, bt, count, inverse, col_scale);
-    else ntt16_launch_od<false>(ctx, bt, count, inverse, col_scale);
+    if (ctx->tune.ntt_tw) ntt16_launch_od<true>(ctx, bt, count, inverse, col_scale, fin);
+    else ntt16_launch_od<false>(ctx, bt, count, inverse, col_scale, fin);
 }
 
-// N = 2^16 forward pass B alone (after a fused first pass), in place on bt.dst
-template <bool OD>
-static void ntt16_pass_b_od(fg_ctx *ctx, const Batch &bt, int count)
-{
-    const auto *fwd = (const ulonglong2 *)ctx->d_fwd;
-    const auto *rows = (const ulonglong2 *)ctx->d_fwd_rows;
-    if (ctx->tune.ntt_rows == 8)
-        ntt16_fwd_b<8, OD><<<dim3(32, count), 128, 0, ctx->stream>>>(bt, ctx->d_primes, fwd, rows);
-    else
-        ntt16_fwd_b<16, OD><<<dim3(16, count), 256, 0, ctx->stream>>>(bt, ctx->d_primes, fwd, rows);
-}
-
-static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool inverse)
+static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool inverse, const Finish *fin = nullptr)
 {
     FG_CHECK(src.per_row == dst.per_row && src.rows == dst.rows, FG_EINVAL, "ntt: shape mismatch");
     if (src.rows == 0 || src.per_row == 0) return;
@@ -1025,12 +1035,13 @@ static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool
     FG_CHECK(count <= 65535, FG_EINVAL, "ntt: more than 65535 limbs in one batch");
     int active = 0;
     for (int v : src.pidx) active += v >= 0;
-    KTimer kt(ctx, "ntt", (double)active * src.rows * ctx->n * 8 * 2);
+    // finishing: ext read as well, and out when it accumulates
+    KTimer kt(ctx, "ntt", (double)active * src.rows * ctx->n * 8 * (fin ? 3 + fin->accumulate : 2));
     if (ctx->log_n < 16) {
-        ntt_small(ctx, bt, count, inverse);
+        ntt_small(ctx, bt, count, inverse, fin);
         return;
     }
-    ntt16_launch(ctx, bt, count, inverse);
+    ntt16_launch(ctx, bt, count, inverse, nullptr, fin);
     check_launch("ntt", 2);
 }
 
@@ -1081,6 +1092,20 @@ void add(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count, const std::
     k_add<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(a, b, c, contiguous(c, count, pidx),
                                                            ctx->d_primes, ctx->n);
     check_launch("add");
+}
+
+void tensor(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *lane, u64 *d1, int n, int nl)
+{
+    KTimer kt(ctx, "tensor", (double)n * nl * ctx->n * 8 * (a == b ? 5 : 7));
+    k_tensor<<<dim3(ctx->n / 256, nl, n), 256, 0, ctx->stream>>>(a, b, lane, d1, nl, ctx->d_primes, ctx->d_pmodq, ctx->n);
+    check_launch("tensor");
+}
+
+void add_part1(fg_ctx *ctx, u64 *u, int E, const u64 *d, int n, int nl)
+{
+    KTimer kt(ctx, "add", (double)n * nl * ctx->n * 8 * 3);
+    k_add_part1<<<dim3(ctx->n / 256, nl, n), 256, 0, ctx->stream>>>(u, E, d, nl, ctx->d_primes, ctx->n);
+    check_launch("add_part1");
 }
 
 void neg(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &pidx)
@@ -1337,7 +1362,7 @@ void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out)
 // ModDown + rescale at N = 2^16 with the conversion fused into w's first
 // NTT pass (see k_moddown_ntt16_a)
 template <bool OD>
-static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls)
+static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls, bool accumulate)
 {
     const int N = ctx->n, l = level, E = ctx->ext(level), npoly = 2 * ncol;
     std::vector<int> pp(E, -1);
@@ -1373,22 +1398,18 @@ static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out
         std::vector<int> pq(l);
         for (int i = 0; i < l; i++) pq[i] = i;
         Batch bw = make_batch(w, l, w, l, l, npoly, pq);
-        KTimer kt(ctx, "ntt", (double)npoly * l * N * 8 * 2 / 2);
-        ntt16_pass_b_od<OD>(ctx, bw, npoly * l);
+        const Finish fin{ext, out, ctx->moddown_rescale_tab(level), E, ls, accumulate ? 1 : 0};
+        KTimer kt(ctx, "ntt", (double)npoly * l * N * 8 * (2 + fin.accumulate));
+        ntt16_pass_b_od<OD>(ctx, bw, npoly * l, &fin);
         check_launch("ntt16_fwd_b");
     }
-    KTimer kt(ctx, "moddown_store", (double)npoly * l * 3 * N * 8);
-    dim3 g3((N / 2 + 255) / 256, l);
-    k_moddown_rescale_finish<<<g3, 256, 0, ctx->stream>>>(ext, E, w, out, ls, npoly, l,
-                                                          ctx->moddown_rescale_tab(level), ctx->d_primes, N);
-    check_launch("moddown_rescale_finish");
 }
 
-void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls)
+void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out, int ls, bool accumulate)
 {
     if (ctx->log_n == 16 && ctx->tune.moddown_fused && level >= 1) {
-        if (ctx->tune.ntt_tw) moddown16_fused<true>(ctx, ext, ncol, level, out, ls);
-        else moddown16_fused<false>(ctx, ext, ncol, level, out, ls);
+        if (ctx->tune.ntt_tw) moddown16_fused<true>(ctx, ext, ncol, level, out, ls, accumulate);
+        else moddown16_fused<false>(ctx, ext, ncol, level, out, ls, accumulate);
         return;
     }
     FG_CHECK(level >= 1, FG_ELEVEL, "rescale needs level >= 1");
@@ -1413,14 +1434,11 @@ void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *ou
     }
     std::vector<int> pq(l);
     for (int i = 0; i < l; i++) pq[i] = i;
+    // the rescaled limbs (ext_i - NTT(w)_i) (P q_l)^-1 straight from the
+    // transform's last pass
     LimbSet ws{w, l, l, npoly, pq};
-    ntt_fwd(ctx, ws, ws);
-    KTimer kt(ctx, "moddown_store", (double)npoly * l * 3 * N * 8);
-    dim3 g3((N / 2 + 255) / 256, l);
-    k_moddown_rescale_finish<<<g3, 256, 0, ctx->stream>>>(ext, E, w, out, ls, npoly, l,
-                                                          ctx->moddown_rescale_tab(level),
-                                                          ctx->d_primes, N);
-    check_launch("moddown_rescale_finish");
+    const Finish fin{ext, out, ctx->moddown_rescale_tab(level), E, ls, accumulate ? 1 : 0};
+    launch_ntt(ctx, ws, ws, false, &fin);
 }
 
 }  // namespace kern

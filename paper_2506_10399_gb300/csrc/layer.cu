@@ -558,7 +558,6 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             bufB[i] = (u64 *)ctx->buf("lane_b" + std::to_string(i), lane_w * 8);
         }
         u64 *acc = (u64 *)ctx->buf("acc", lane_w * 8);
-        u64 *acc_new = (u64 *)ctx->buf("acc_new", lane_w * 8);
 
         // ---- Inter-CA (the client sent one copy of X per neighbour slot k):
         // Z_k = X_k W for every copy, then out = sum_k mask_k (x) Z_k, rescale
@@ -577,13 +576,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             kern::rescale_ntt(ctx, acc, LS, Fp * 2, l1);
             const int level = l1 - 1, nlo = level + 1;
             FG_CHECK(level == pl->out_level, FG_ELEVEL, "plan output level mismatch");
-            std::vector<int> pidx(LS, -1);
-            for (int i = 0; i < nlo; i++) pidx[i] = i;
-            kern::LimbSet as{acc, LS, LS, Fp * 2, pidx};
-            kern::ntt_inv(ctx, as, as);
             const size_t out_w = (size_t)Fp * 2 * nlo * N;
             u64 *o = is_dev(out_cts) ? out_cts : (u64 *)ctx->buf("layer_out", out_w * 8);
-            kern::copy_limbs(ctx, acc, LS, o, nlo, Fp * 2, nlo);
+            kern::LimbSet as{acc, LS, nlo, Fp * 2, iota(nlo)}, os{o, nlo, nlo, Fp * 2, iota(nlo)};
+            kern::ntt_inv(ctx, as, os);
             if (o != out_cts)
                 CUDA_TRY(cudaMemcpyAsync(out_cts, o, out_w * 8, cudaMemcpyDeviceToHost, ctx->stream));
             if (sync) {
@@ -631,7 +627,7 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             kern::rescale_ntt(ctx, Za, nl0, Fp * 2, l0);
             kern::copy_limbs(ctx, Za, nl0, bufA[0], LS, Fp * 2, LS);
             u64 *digits = (u64 *)ctx->buf("digits", (size_t)Fp * ctx->n_digits(l1) * ctx->ext(l1) * N * 8);
-            u64 *tmp = acc_new;
+            u64 *tmp = (u64 *)ctx->buf("acc_new", lane_w * 8);
             for (int k : pl->comb_rots) {
                 kern::modup(ctx, bufA[0], LS, Fp, l1, digits);
                 kern::rotate(ctx, keys->get(((k % M) + M) % M), bufA[0], LS, Fp, l1, digits, tmp, LS);
@@ -761,15 +757,8 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
             for (int x = 0; x < g.n_out; x++)
                 kern::moddown_rescale_to_lane(ctx, ext[x], Fp, level, (*outb)[x], LS);
             if (any_acc) {
-                kern::moddown_rescale_to_lane(ctx, ext[g.n_out], Fp, level, acc_new, LS);
-                if (have_acc) {
-                    std::vector<int> pidx(LS, -1);
-                    for (int i = 0; i < level; i++) pidx[i] = i;
-                    kern::add(ctx, acc, acc_new, acc, Fp * 2 * LS, pidx);
-                } else {
-                    std::swap(acc, acc_new);
-                    have_acc = true;
-                }
+                kern::moddown_rescale_to_lane(ctx, ext[g.n_out], Fp, level, acc, LS, have_acc);
+                have_acc = true;
             }
             std::swap(in, outb);
             level--;
@@ -779,13 +768,10 @@ static void layer_exec(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, cons
 
         // ---- 3. back to the coefficient domain, compact [Fp][2][level+1][N]
         const int nlo = level + 1;
-        std::vector<int> pidx(LS, -1);
-        for (int i = 0; i < nlo; i++) pidx[i] = i;
-        kern::LimbSet as{acc, LS, LS, Fp * 2, pidx};
-        kern::ntt_inv(ctx, as, as);
         const size_t out_w = (size_t)Fp * 2 * nlo * N;
         u64 *o = is_dev(out_cts) ? out_cts : (u64 *)ctx->buf("layer_out", out_w * 8);
-        kern::copy_limbs(ctx, acc, LS, o, nlo, Fp * 2, nlo);
+        kern::LimbSet as{acc, LS, nlo, Fp * 2, iota(nlo)}, os{o, nlo, nlo, Fp * 2, iota(nlo)};
+        kern::ntt_inv(ctx, as, os);
         if (o != out_cts)
             CUDA_TRY(cudaMemcpyAsync(out_cts, o, out_w * 8, cudaMemcpyDeviceToHost, ctx->stream));
         if (sync) {

@@ -20,6 +20,8 @@
 // event overhead (before / now): 608 limbs of N = 2^15 305 / 209, of 2^14 138 /
 // 103, of 2^13 72 / 58, of 2^12 41 / 31; 8 limbs 17 / 15, 19 / 15, 16 / 15, 16 /
 // 13.
+#include <type_traits>
+
 #include "ntt.cuh"
 
 namespace {
@@ -182,12 +184,6 @@ struct RowPass {
             v[m + 1] = a.y;
         }
     }
-    static __device__ __forceinline__ void store(const u64 (&v)[16], u64 *p, int t)
-    {
-#pragma unroll
-        for (int m = 0; m < 16; m += 2)
-            *reinterpret_cast<ulonglong2 *>(p + Last::elem(t, m / Last::R, m % Last::R)) = make_ulonglong2(v[m], v[m + 1]);
-    }
 };
 
 // blocks per SM to budget the registers for: 64 to 80 a thread
@@ -195,10 +191,10 @@ template <int LOGN, int LS>
 constexpr int row_blocks() { return RowPass<LOGN, LS>::THREADS >= 512 ? 2 : RowPass<LOGN, LS>::THREADS >= 256 ? 3 : 6; }
 
 // first / only pass over rows.  FIRST (whole limbs): reads src, else in place.
-template <int LOGN, int LS>
+template <int LOGN, int LS, bool FIN>
 __global__ void __launch_bounds__(RowPass<LOGN, LS>::THREADS, row_blocks<LOGN, LS>())
 ntt_rows_fwd(const __grid_constant__ Batch bt, const PrimeC *__restrict__ primes, const ulonglong2 *__restrict__ tw,
-             const ulonglong2 *__restrict__ tw_last)
+             const ulonglong2 *__restrict__ tw_last, const Finish fin)
 {
     typedef RowPass<LOGN, LS> W;
     typedef Round<LS, 0> A;
@@ -211,22 +207,26 @@ ntt_rows_fwd(const __grid_constant__ Batch bt, const PrimeC *__restrict__ primes
     const PrimeC P = primes[pi];
     const u64 *src = (LS == LOGN ? bt.src + ((size_t)lrow * bt.src_stride + col) * N
                                  : bt.dst + ((size_t)lrow * bt.dst_stride + col) * N) + ((size_t)row << LS);
-    u64 *dst = bt.dst + ((size_t)lrow * bt.dst_stride + col) * N + ((size_t)row << LS);
+    u64 *dst = bt.dst + ((size_t)lrow * bt.dst_stride + col) * N;
     u64 v[16];
 #pragma unroll
     for (int m = 0; m < 16; m++) v[m] = src[A::elem(t, m / A::R, m % A::R)];
     const Tw<LS, W::S0> w{tw + (size_t)pi * N, row};
     const ulonglong2 *last = tw_last + (size_t)pi * N + ((size_t)row << LS >> Rounds<LS>::r[Rounds<LS>::n - 1]) + t;
+    const auto put = [&](auto lazy) {   // the last round's groups are contiguous
+#pragma unroll
+        for (int m = 0; m < 16; m += 2)
+            put_pair<decltype(lazy)::value, FIN>(
+                v[m], v[m + 1], dst, ((size_t)row << LS) + W::Last::elem(t, m / W::Last::R, m % W::Last::R), fin, lrow, col,
+                N, P);
+    };
     if (P.q < (1ull << 47)) {
         fwd_all<LS, W::S0, true>(v, t, s, W::pad(), w, last, W::NB, P.q);
-#pragma unroll
-        for (int m = 0; m < 16; m++) v[m] = reduce_word(v[m], P);
+        put(std::true_type());
     } else {
         fwd_all<LS, W::S0, false>(v, t, s, W::pad(), w, last, W::NB, P.q);
-#pragma unroll
-        for (int m = 0; m < 16; m++) v[m] = reduce8(v[m], P.q);
+        put(std::false_type());
     }
-    W::store(v, dst, t);
 }
 
 template <int LOGN, int LS>
@@ -321,27 +321,37 @@ __global__ void k_last_table(const ulonglong2 *__restrict__ tab, ulonglong2 *las
     last[(size_t)blockIdx.y * N + k] = tab[(size_t)blockIdx.y * N + (1 << (log_n - r + st)) + ((size_t)b << st) + x];
 }
 
-template <int LOGN, int LS, bool INV>
-void launch_rows(fg_ctx *ctx, const Batch &bt, int count)
+template <int LOGN, int LS, bool FIN>
+void launch_rows_fwd(fg_ctx *ctx, const Batch &bt, int count, const Finish &fin)
 {
     typedef RowPass<LOGN, LS> W;
     const size_t sm = (size_t)W::ROWS * W::PADDED * 8;
     const dim3 g((1 << (LOGN - LS)) / W::ROWS, count);
-    if (INV) {
-        if (sm > 48 * 1024)
-            CUDA_TRY(cudaFuncSetAttribute(ntt_rows_inv<LOGN, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        ntt_rows_inv<LOGN, LS><<<g, W::THREADS, sm, ctx->stream>>>(bt, ctx->d_primes, (const ulonglong2 *)ctx->d_inv,
-                                                                  (const ulonglong2 *)ctx->d_inv_last, ctx->d_ninv);
-    } else {
-        if (sm > 48 * 1024)
-            CUDA_TRY(cudaFuncSetAttribute(ntt_rows_fwd<LOGN, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        ntt_rows_fwd<LOGN, LS><<<g, W::THREADS, sm, ctx->stream>>>(bt, ctx->d_primes, (const ulonglong2 *)ctx->d_fwd,
-                                                                  (const ulonglong2 *)ctx->d_fwd_last);
+    if (sm > 48 * 1024)
+        CUDA_TRY(cudaFuncSetAttribute(ntt_rows_fwd<LOGN, LS, FIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ntt_rows_fwd<LOGN, LS, FIN><<<g, W::THREADS, sm, ctx->stream>>>(
+        bt, ctx->d_primes, (const ulonglong2 *)ctx->d_fwd, (const ulonglong2 *)ctx->d_fwd_last, fin);
+}
+
+template <int LOGN, int LS>
+void launch_rows(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin)
+{
+    if (!inverse) {
+        if (fin) launch_rows_fwd<LOGN, LS, true>(ctx, bt, count, *fin);
+        else launch_rows_fwd<LOGN, LS, false>(ctx, bt, count, Finish());
+        return;
     }
+    typedef RowPass<LOGN, LS> W;
+    const size_t sm = (size_t)W::ROWS * W::PADDED * 8;
+    const dim3 g((1 << (LOGN - LS)) / W::ROWS, count);
+    if (sm > 48 * 1024)
+        CUDA_TRY(cudaFuncSetAttribute(ntt_rows_inv<LOGN, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ntt_rows_inv<LOGN, LS><<<g, W::THREADS, sm, ctx->stream>>>(bt, ctx->d_primes, (const ulonglong2 *)ctx->d_inv,
+                                                              (const ulonglong2 *)ctx->d_inv_last, ctx->d_ninv);
 }
 
 template <int LOGN>
-void two_passes(fg_ctx *ctx, const Batch &bt, int count, bool inverse)
+void two_passes(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin)
 {
     const dim3 g((1 << (LOGN - kColS)) / kCols, count);
     Batch b2 = bt;
@@ -349,18 +359,11 @@ void two_passes(fg_ctx *ctx, const Batch &bt, int count, bool inverse)
     b2.src_stride = b2.dst_stride;
     if (!inverse) {
         ntt_cols_fwd<LOGN><<<g, 128, 0, ctx->stream>>>(bt, ctx->d_primes, (const ulonglong2 *)ctx->d_fwd);
-        launch_rows<LOGN, LOGN - kColS, false>(ctx, b2, count);
+        launch_rows<LOGN, LOGN - kColS>(ctx, b2, count, false, fin);
     } else {
-        launch_rows<LOGN, LOGN - kColS, true>(ctx, bt, count);
+        launch_rows<LOGN, LOGN - kColS>(ctx, bt, count, true, nullptr);
         ntt_cols_inv<LOGN><<<g, 128, 0, ctx->stream>>>(b2, ctx->d_primes, (const ulonglong2 *)ctx->d_inv, ctx->d_ninv);
     }
-}
-
-template <int LOGN>
-void one_pass(fg_ctx *ctx, const Batch &bt, int count, bool inverse)
-{
-    if (inverse) launch_rows<LOGN, LOGN, true>(ctx, bt, count);
-    else launch_rows<LOGN, LOGN, false>(ctx, bt, count);
 }
 
 }  // namespace
@@ -384,23 +387,23 @@ void ntt_last_tables(fg_ctx *ctx)
     CUDA_TRY(cudaStreamSynchronize(ctx->stream));
 }
 
-void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse)
+void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin)
 {
     bool one = ctx->log_n <= 12;
     switch (ctx->log_n) {
-    case 10: one_pass<10>(ctx, bt, count, inverse); break;
-    case 11: one_pass<11>(ctx, bt, count, inverse); break;
-    case 12: one_pass<12>(ctx, bt, count, inverse); break;
+    case 10: launch_rows<10, 10>(ctx, bt, count, inverse, fin); break;
+    case 11: launch_rows<11, 11>(ctx, bt, count, inverse, fin); break;
+    case 12: launch_rows<12, 12>(ctx, bt, count, inverse, fin); break;
     case 13: {
         // one block a limb leaves most SMs idle below 100 limbs (us: one pass /
         // two, 8 limbs 14.8 / 9.5, 64 14.9 / 12.0, 128 14.6 / 17.6)
         one = count >= 100;
-        if (one) one_pass<13>(ctx, bt, count, inverse);
-        else two_passes<13>(ctx, bt, count, inverse);
+        if (one) launch_rows<13, 13>(ctx, bt, count, inverse, fin);
+        else two_passes<13>(ctx, bt, count, inverse, fin);
         break;
     }
-    case 14: two_passes<14>(ctx, bt, count, inverse); break;
-    case 15: two_passes<15>(ctx, bt, count, inverse); break;
+    case 14: two_passes<14>(ctx, bt, count, inverse, fin); break;
+    case 15: two_passes<15>(ctx, bt, count, inverse, fin); break;
     default: throw fg_error(FG_EINVAL, "ntt: unsupported ring degree");
     }
     const cudaError_t e = cudaGetLastError();

@@ -72,5 +72,40 @@ __device__ __forceinline__ void gs_round(u64 *v, TW tw, u64 q, u64 q4, int k0)
     }
 }
 
-// N = 2^10 .. 2^15 (ntt.cu)
-void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse);
+// What a forward transform may do with its results w instead of storing them:
+// out_i (+)= (ext_i - w_i) c_i mod q_i for limb i of every row, c with its Shoup
+// companion at c[2 i].  ext and out have E and ls limbs a row.
+struct Finish {
+    const u64 *ext;
+    u64 *out;
+    const u64 *c;
+    int E, ls, accumulate;
+};
+
+// Two neighbouring results of one limb (row, col), at word offset pos: reduced
+// and stored at d + pos, or finished.  w is lazy: below 65 q (LAZY) or 8 q.
+template <bool LAZY, bool FIN>
+__device__ __forceinline__ void put_pair(u64 w0, u64 w1, u64 *d, size_t pos, const Finish &f, int row, int col, int N,
+                                         const PrimeC &P)
+{
+    ulonglong2 *o;
+    ulonglong2 r;
+    if (FIN) {
+        const u64 q = P.q, c = f.c[2 * col], cs = f.c[2 * col + 1], up = (LAZY ? 65 : 8) * q;
+        const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(f.ext + ((size_t)row * f.E + col) * N + pos);
+        r = make_ulonglong2(shoup_mul(e.x + up - w0, c, cs, q), shoup_mul(e.y + up - w1, c, cs, q));
+        o = reinterpret_cast<ulonglong2 *>(f.out + ((size_t)row * f.ls + col) * N + pos);
+        if (f.accumulate) {
+            const ulonglong2 b = *o;
+            r = make_ulonglong2(add_mod(r.x, b.x, q), add_mod(r.y, b.y, q));
+        }
+    } else {
+        r = LAZY ? make_ulonglong2(reduce_word(w0, P), reduce_word(w1, P))
+                 : make_ulonglong2(reduce8(w0, P.q), reduce8(w1, P.q));
+        o = reinterpret_cast<ulonglong2 *>(d + pos);
+    }
+    *o = r;
+}
+
+// N = 2^10 .. 2^15 (ntt.cu); fin: forward only
+void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin = nullptr);
