@@ -6,9 +6,9 @@
 // exchanges (radix-16 rounds, or two radix-8 groups).
 //   * Up to N = 2^13 one block transforms a whole limb: one launch and one
 //     read and write of global memory per transform.
-//   * N = 2^14, 2^15 and small batches at 2^13 take two passes: the first seven
-//     stages on 128-row columns (16 columns a block), the rest inside rows of
-//     64, 128 or 256 (2048 elements a block).
+//   * N = 2^14, 2^15 and small batches at 2^12 and 2^13 take two passes: the first
+//     seven stages on 128-row columns (16 columns a block), the rest inside rows
+//     of 32 to 256 (2048 elements a block).
 // The last round's twiddles, one set per thread, come from a table of their own
 // (d_fwd_last, d_inv_last: [prime][group of the round][thread of the limb]) so
 // that a warp reads consecutive entries.
@@ -28,6 +28,7 @@ namespace {
 
 // stages per round of a transform of 2^LS elements
 template <int LS> struct Rounds;
+template <> struct Rounds<5>  { static constexpr int n = 2, r[4] = {1, 4, 0, 0}; };
 template <> struct Rounds<6>  { static constexpr int n = 2, r[4] = {3, 3, 0, 0}; };
 template <> struct Rounds<7>  { static constexpr int n = 2, r[4] = {4, 3, 0, 0}; };
 template <> struct Rounds<8>  { static constexpr int n = 2, r[4] = {4, 4, 0, 0}; };
@@ -374,7 +375,7 @@ void ntt_last_tables(fg_ctx *ctx)
     switch (ctx->log_n) {
     case 10: r = Rounds<10>::r[2]; break;
     case 11: r = Rounds<11>::r[2]; break;
-    case 12: r = Rounds<12>::r[2]; break;
+    case 12: r = Rounds<12>::r[2]; break;   // = Rounds<5>::r[1]
     case 13: r = Rounds<13>::r[3]; break;   // = Rounds<6>::r[1]
     case 14: r = Rounds<7>::r[1]; break;
     case 15: r = Rounds<8>::r[1]; break;
@@ -389,11 +390,17 @@ void ntt_last_tables(fg_ctx *ctx)
 
 void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin)
 {
-    bool one = ctx->log_n <= 12;
+    bool one = ctx->log_n <= 11;
     switch (ctx->log_n) {
     case 10: launch_rows<10, 10>(ctx, bt, count, inverse, fin); break;
     case 11: launch_rows<11, 11>(ctx, bt, count, inverse, fin); break;
-    case 12: launch_rows<12, 12>(ctx, bt, count, inverse, fin); break;
+    case 12:
+        // as at 2^13, below 80 limbs: a rotation (3 to 12 limbs a transform, six
+        // transforms) 118 / 111 us; 96 limbs 12.2 / 13.8 us
+        one = count >= 80;
+        if (one) launch_rows<12, 12>(ctx, bt, count, inverse, fin);
+        else two_passes<12>(ctx, bt, count, inverse, fin);
+        break;
     case 13: {
         // one block a limb leaves most SMs idle below 100 limbs (us: one pass /
         // two, 8 limbs 14.8 / 9.5, 64 14.9 / 12.0, 128 14.6 / 17.6)

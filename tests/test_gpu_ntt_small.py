@@ -1,6 +1,6 @@
 """Transforms at N = 2^10 .. 2^15: every ring degree, primes below and above
-2^47 (lazy and reduced butterflies), one limb, the two sides of the batch size
-where N = 2^13 changes from two passes to one, limbs left alone in between;
+2^47 (lazy and reduced butterflies), one limb, the two sides of the batch sizes
+where N = 2^12 and 2^13 change from two passes to one, limbs left alone in between;
 forward then inverse, and products against the oracle's negacyclic product."""
 import numpy as np
 import pytest
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("log_n", range(10, 16))
-@pytest.mark.parametrize("rows", [1, 24, 25, 40])
+@pytest.mark.parametrize("rows", [1, 19, 20, 24, 25, 40])
 def test_round_trip_and_product(log_n, rows):
     import torch
     if not torch.cuda.is_available():
