@@ -386,8 +386,8 @@ int fg_gcn_layer_axw_seeded(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pla
  * (held in registers per round, or loaded where used at one more CTA per
  * SM), the key switch's
  * register budget (its launch bound at the default or one CTA per SM
- * fewer) and the output count from which a group-MAC CTA runs three thread
- * groups (7, 4 or 13); fg_batch_tuning reports the choice.  Every
+ * fewer or more) and the output count from which a group-MAC CTA of the form
+ * for more than six outputs runs three thread groups (7, 4 or 13); fg_batch_tuning reports the choice.  Every
  * configuration computes the same words, and every query runs the kernels
  * of fg_gcn_layer_axw, so the outputs are the same word for word.  opts
  * NULL = {0, 1, 0}.  Host buffers: FG_EINVAL. */
@@ -411,10 +411,11 @@ int fg_gcn_layer_batch_seeded(fg_ctx *ctx, const fg_keys *keys, const fg_plan *c
                               int *streams_used);
 /* The batched form's launch configuration: cfg = {NTT pass-A columns, NTT
  * pass-B rows, NTT twiddles loaded where used (0/1), key-switch registers
- * (0 default, 1 one CTA per SM fewer, 2 keys in shared memory), key-switch column launches (1/2), fused ModUp
- * (0/1), fused ModDown (0/1), group-MAC three-group threshold, group-MAC
- * registers for three CTAs per SM (0/1), group-MAC products below 2^46 in
- * Karatsuba's form, three multiplies instead of four (1, the default, or 0)}; ms[0..*n) the
+ * (0 default, 1 one CTA per SM fewer, 2 one more), key-switch column launches
+ * (1/2), fused ModUp (0/1), fused ModDown (0/1), and for groups of more than
+ * six outputs: group-MAC three-group threshold, group-MAC registers for three
+ * CTAs per SM (0/1), group-MAC products below 2^46 in Karatsuba's form, three
+ * multiplies instead of four (1, the default, or 0)}; ms[0..*n) the
  * batch pass time of each configuration tried (the default first), at most
  * cap entries.  Before any tuned batch call cfg holds the context's
  * configuration and *n = 0. */

@@ -8,10 +8,10 @@
 //      rescale, log t rotate-and-sum steps;
 //   2. SpIntra-CA groups: per input lane one ModUp of c1 (hoisted, shared by
 //      all its rotation amounts), per rotation one key-switching inner
-//      product and ModDown whose epilogue multiplies the rotated ciphertext
-//      by every mask that uses it and adds it into the output lanes and the
-//      accumulator; kept values (rotation 0) are masked the same way; then
-//      every output and the group's accumulator are rescaled and the running
+//      product over the extended primes; every rotation and kept value
+//      (rotation 0) is multiplied by each mask that uses it and summed into
+//      the output lanes and the accumulator, still extended; then every
+//      output takes one ModDown with its rescale, and the running
 //      accumulator, dropped one limb, receives the group's arrivals;
 //   3. the accumulator returns to the coefficient domain.
 // All F' output columns share the plan, so every kernel runs over all
