@@ -204,6 +204,8 @@ static ConvTab make_conv(const fg_ctx &c, const std::vector<int> &in_p, const st
         for (int j = 0; j < T.n_in; j++) B = hm::mulmod(B, c.primes[in_p[j]] % p, p);
         const u64 nb = hm::to_mont((p - B) % p, p);
         T.negb[t] = (nb & 0x3FFFFFFFull) | ((nb >> 30) << 32);
+        const u64 b = hm::to_mont(B, p);
+        T.posb[t] = (b & 0x3FFFFFFFull) | ((b >> 30) << 32);
     }
     return T;
 }
@@ -379,13 +381,14 @@ const u64 *fg_ctx::moddown_rescale_half_tab(int level)
 {
     auto it = mdr_half_tabs.find(level);
     if (it != mdr_half_tabs.end()) return it->second;
-    std::vector<u64> h(level + 1);
+    std::vector<u64> h(2 * (level + 1));   // [H]_{q_i}, then [-H - 8 P]_{q_i} in Montgomery form
     const u64 hl = (primes[level] - 1) / 2;
     for (int i = 0; i <= level; i++) {
         const u64 q = primes[i];
         u64 P = 1;
         for (int k = 0; k < np; k++) P = hm::mulmod(P, primes[nq + k] % q, q);
         h[i] = hm::mulmod(P, hl % q, q);
+        h[level + 1 + i] = hm::to_mont((2 * q - h[i] - hm::mulmod(P, 8, q)) % q, q);
     }
     u64 *d = nullptr;
     CUDA_TRY(cudaMalloc(&d, h.size() * 8));

@@ -86,6 +86,7 @@ struct ConvTab {
     u64 hinv[8], hinv_s[8];   // (B/b_k)^-1 mod b_k and its Shoup companion
     u64 hmod[8][72];          // (B/b_k) mod out prime, Montgomery form, 30-bit halves (lo | hi << 32)
     u64 negb[72];             // -B mod out prime, same form (the centred conversion's correction)
+    u64 posb[72];             // B mod out prime, same form
 };
 
 // kernel launch configurations that compute the same words and differ in

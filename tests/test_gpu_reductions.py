@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 SETS = [
     (5, 1, 1, 45), (6, 1, 1, 46), (7, 1, 1, 45), (8, 1, 1, 47), (9, 1, 1, 60),   # digits
-    (7, 6, 6, 45), (8, 7, 7, 60), (9, 8, 7, 46),                                 # primes a digit, special primes
+    (7, 6, 6, 45), (8, 7, 7, 60), (9, 8, 7, 46), (4, 2, 2, 60), (6, 5, 5, 45),   # primes a digit, special primes
 ]
 
 
