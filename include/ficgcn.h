@@ -476,7 +476,8 @@ int fg_poly_mul_noalloc(fg_ctx *ctx, const uint64_t *a, const uint64_t *b, int l
  * [count][N] whose limb c is taken modulo prime index prime_idx[c %
  * period] (0..n_q-1 for q_i, n_q.. for p_k).  The forward output order is
  * private to the library; inverse(forward(x)) = x.  For throughput
- * measurements. */
+ * measurements.  Data that is not 16-byte aligned is taken too, at the price
+ * of a copy through the context's workspace. */
 int fg_ntt(fg_ctx *ctx, uint64_t *data, int count, const int *prime_idx, int period,
            int inverse);
 

@@ -1190,8 +1190,24 @@ int fg_ntt(fg_ctx *ctx, uint64_t *data, int count, const int *prime_idx, int per
     std::vector<int> pid(prime_idx, prime_idx + period);
     for (int p : pid) FG_CHECK(p >= 0 && p < ctx->nq + ctx->np, FG_EINVAL, "bad prime index");
     kern::LimbSet s{data, period, period, count / period, pid};
-    if (inverse) kern::ntt_inv(ctx, s, s);
-    else kern::ntt_fwd(ctx, s, s);
+    if ((uintptr_t)data % 16 == 0) {
+        if (inverse) kern::ntt_inv(ctx, s, s);
+        else kern::ntt_fwd(ctx, s, s);
+    } else {
+        // The forward transform stores pairs of words and the inverse loads
+        // pairs, so that side goes through a workspace; the other side of each
+        // reads or writes single words and stays on the caller's buffer.
+        const size_t bytes = (size_t)count * ctx->n * 8;
+        u64 *w = (u64 *)ctx->buf("ntt_pairs", bytes);
+        kern::LimbSet ws{w, period, period, count / period, pid};
+        if (inverse) {
+            CUDA_TRY(cudaMemcpyAsync(w, data, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+            kern::ntt_inv(ctx, ws, s);
+        } else {
+            kern::ntt_fwd(ctx, s, ws);
+            CUDA_TRY(cudaMemcpyAsync(data, w, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+        }
+    }
     sync(ctx);
     API_CATCH(ctx)
 }
