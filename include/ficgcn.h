@@ -115,6 +115,12 @@ int fg_ctx_launch_count(const fg_ctx *ctx, int64_t *launches);
  * buffers its calls grow on demand and keep for reuse); later calls
  * allocate again.  Keys, plans and tables stay. */
 int fg_ctx_release_workspace(fg_ctx *ctx);
+/* Polls (about 4 us each; 2^18, a second, at first) after which a wait inside
+ * a kernel gives up: the kernel ends, the call returns FG_ETIMEOUT and its
+ * outputs are undefined; the context stays usable.  0: every such wait gives
+ * up at once, so that a caller can try its handling of FG_ETIMEOUT.  Graphs
+ * captured by fg_gcn_layer_batch keep the limit they were captured with. */
+int fg_ctx_set_wait_tries(fg_ctx *ctx, uint32_t tries);
 
 /* ---------------------------------------------------------------- client */
 

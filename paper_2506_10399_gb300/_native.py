@@ -99,6 +99,7 @@ SIGS = {
                                           P(BatchOpts), c_void_p, P(c_int)]),
     "fg_ctx_set_tuning": (c_int, [c_void_p, c_void_p]),
     "fg_ctx_release_workspace": (c_int, [c_void_p]),
+    "fg_ctx_set_wait_tries": (c_int, [c_void_p, ctypes.c_uint32]),
     "fg_batch_tuning": (c_int, [c_void_p, c_void_p, c_void_p, c_int, P(c_int)]),
     "fg_gcn_layer_axw": (c_int, [c_void_p, c_void_p, c_void_p, c_void_p, c_int, c_void_p, c_int,
                                  P(c_int), P(c_double)]),

@@ -143,6 +143,13 @@ void fg_ctx::check_waits()
     throw fg_error(FG_ETIMEOUT, "a kernel's bounded wait ran out");
 }
 
+extern "C" int fg_ctx_set_wait_tries(fg_ctx *ctx, uint32_t tries)
+{
+    if (!ctx) return FG_EINVAL;
+    ctx->wait_tries = tries;
+    return FG_OK;
+}
+
 extern "C" int fg_ctx_release_workspace(fg_ctx *ctx)
 {
     if (!ctx) return FG_EINVAL;

@@ -57,6 +57,7 @@ constexpr int kGroup = kProd / 2;  // two groups of warps cut alternate stages
 // then up to two of the other group): with three slots or more its wait for an
 // empty slot is never more than one phase ahead of the barrier.
 static_assert(kStages >= 3, "slots");
+constexpr u32 kWaitTries = fg_ctx::kWaitTries;
 constexpr int kMaxCols = 8192;     // columns per launch: the 64-bit sums hold 64 segments
 constexpr int kDigBytes = kTileX * kKB * 2;                        // one digit of X in a stage
 constexpr int kStageBytes = 8 * kDigBytes + 8 * 16 * kKB * 2;      // 8 digits of X, 8 of c
@@ -86,23 +87,33 @@ __device__ __forceinline__ void mbar_arrive_tx(u32 bar, u32 bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// Waits for the phase of the given parity.  Every wait is bounded: after
-// kWaitTries polls, or once another role of the block has given up, it sets
-// the block's stop flag and returns false, and the role leaves its loop.
-constexpr u32 kWaitTries = 1u << 23;
-__device__ __forceinline__ bool mbar_wait(u32 bar, u32 parity, volatile int *stop)
+__device__ __forceinline__ bool mbar_poll(u32 bar, u32 parity)
 {
-    for (u32 n = 0; n < kWaitTries; n++) {
-        u32 ok;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
+    u32 ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok;
+}
+// Waits for the phase of the given parity.  Every wait is bounded: after
+// `tries` polls, or once another role of the block has given up, it sets
+// the block's stop flag and returns false, and the role leaves its loop.
+__device__ __forceinline__ bool mbar_wait(u32 bar, u32 parity, volatile int *stop, u32 tries)
+{
+    for (u32 n = 0; n < tries; n++) {
+        if (mbar_poll(bar, parity)) return true;
         if (*stop) return false;
     }
     *stop = 1;
     return false;
+}
+// The same once a role has given up, for what is still under way: always with
+// the default limit, and nothing to report.
+__device__ __forceinline__ void mbar_drain(u32 bar, u32 parity)
+{
+    for (u32 n = 0; n < kWaitTries; n++)
+        if (mbar_poll(bar, parity)) return;
 }
 
 // shared-memory matrix descriptor: K-major, no swizzle; lbo: bytes between
@@ -186,6 +197,7 @@ struct CombArgs {
     int *err;
     int Fp, nl, N, z_ls, nj, dc, tiles;
     int f0, f1, kb_all, corr0, corr1, corr_blocks, accumulate;
+    u32 tries;                  // polls after which a wait gives up
     uint8_t da[64];             // digits of X by limb
     CUtensorMap map;            // X as [columns][part x limb][coefficients]
 };
@@ -211,6 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
     __shared__ __align__(8) u64 bars[2 * kStages + 4 + 2 * kRaw];
     __shared__ u32 tmem_base_s;
     __shared__ volatile int stop;
+    __shared__ u32 cut_end[2];   // stages up to which each group of cutting warps has issued digit copies
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const u32 full = smem_u32(bars), empty = full + 8 * kStages, acc_full = empty + 8 * kStages,
               acc_empty = acc_full + 16, raw_full = acc_empty + 16, raw_empty = raw_full + 8 * kRaw;
@@ -244,6 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
     const int nkb = (A.f1 - A.f0 + kKB - 1) / kKB;   // stages per tile
     constexpr int kbs = kSeg / kKB;                  // stages per segment
     const u32 bbytes = (u32)A.dc * 16 * kKB * 2;
+    u32 it = 0, seg = 0;   // stages and segments of the block so far
 
     if (warp < 8) {
         // ---- accumulators -> 64-bit sums -> Z
@@ -254,7 +268,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         mbar_arrive(acc_empty);
         mbar_arrive(acc_empty + 8);
-        u32 seg = 0;
         bool ok = true;
         Tile T;
         for (T.set(A, blockIdx.x); T.t < A.tiles && ok; T.set(A, T.t + gridDim.x)) {
@@ -266,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
                 for (int j = 0; j < 8; j++) g[r][j] = 0;
             for (int kb = 0; kb < nkb && ok; kb += kbs, seg++) {
                 const u32 b = seg & 1, ta = tq + b * 256;
-                ok = mbar_wait(acc_full + 8 * b, seg >> 1 & 1, &stop);
+                ok = mbar_wait(acc_full + 8 * b, seg >> 1 & 1, &stop, A.tries);
                 ok = __all_sync(0xFFFFFFFFu, ok);   // the tcgen05 loads are warp-wide
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -323,8 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
         // ---- words of X -> digits
         const int x = (tid - kEpi) % kGroup;               // kGroup == kTileX
         const u32 grp = (u32)(tid - kEpi) / kGroup;
-        u32 it = 0;        // stages of the block so far; the group cuts those with it % 2 == grp
-        u32 mine = ~0u;    // the last of them
+        u32 mine = 0;      // the group cuts the stages with it % 2 == grp; one past the last of them
         bool ok = true;
         Tile T;
         for (T.set(A, blockIdx.x); T.t < A.tiles && ok; T.set(A, T.t + gridDim.x)) {
@@ -332,14 +344,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
             for (int kb = 0; kb < nkb; kb++, it++) {
                 if ((it & 1) != grp) continue;
                 const u32 s = it % kStages, rs = it % kRaw;
-                ok = mbar_wait(raw_full + 8 * rs, it / kRaw & 1, &stop);
-                if (ok && it >= kStages) ok = mbar_wait(empty + 8 * s, (it / kStages - 1) & 1, &stop);
+                ok = mbar_wait(raw_full + 8 * rs, it / kRaw & 1, &stop, A.tries);
+                if (ok && it >= kStages) ok = mbar_wait(empty + 8 * s, (it / kStages - 1) & 1, &stop, A.tries);
                 if (!ok) break;
                 if (x == 0) {
                     mbar_arrive_tx(full + 8 * s, bbytes);
                     bulk_copy(smem0 + s * kStageBytes + 8 * kDigBytes, dig + (size_t)kb * bbytes, bbytes, full + 8 * s);
                 }
-                mine = it;
+                mine = it + 1;
                 const unsigned char *src = sm + rs * kRawBytes + x * 8;
                 unsigned char *dst = dig0 + s * kStageBytes + x * 16;
                 u32 lo[2][8], hi[2][8];
@@ -360,46 +372,34 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
                 }
             }
         }
-        // leaving early: a bulk copy may still be under way into this block's
-        // shared memory; wait for it (bounded) before the block can end
-        if (!ok && x == 0 && mine != ~0u) {
-            int never = 0;
-            mbar_wait(full + 8 * (mine % kStages), mine / kStages & 1, &never);
-        }
+        if (x == 0) cut_end[grp] = mine;
     } else if (warp == 17) {
         // ---- words of X: columns past the last arrive as zeros
         if (lane == 0) {
-            u32 it = 0;
             bool ok = true;
             Tile T;
             for (T.set(A, blockIdx.x); T.t < A.tiles && ok; T.set(A, T.t + gridDim.x)) {
                 for (int kb = 0; kb < nkb; kb++, it++) {
                     const u32 rs = it % kRaw;
-                    if (it >= kRaw) ok = mbar_wait(raw_empty + 8 * rs, (it / kRaw - 1) & 1, &stop);
+                    if (it >= kRaw) ok = mbar_wait(raw_empty + 8 * rs, (it / kRaw - 1) & 1, &stop, A.tries);
                     if (!ok) break;
                     mbar_arrive_tx(raw_full + 8 * rs, kRawBytes);
                     tma_load(raw0 + rs * kRawBytes, &A.map, T.xb * kTileX, T.p * A.nl + T.i, A.f0 + kb * kKB,
                              raw_full + 8 * rs);
                 }
             }
-            if (!ok)   // leaving early: the copies under way, bounded
-                for (u32 k = it > kRaw ? it - kRaw : 0; k < it; k++) {
-                    int never = 0;
-                    mbar_wait(raw_full + 8 * (k % kRaw), k / kRaw & 1, &never);
-                }
         }
         __syncwarp();
     } else {
         // ---- the products
         const u32 idesc = 1u << 4 | (u32)(2 * A.dc) << 17 | (u32)(kTileX >> 4) << 24;   // f32 += f16 f16, N = 16 Dc
-        u32 it = 0, seg = 0;   // stages, segments
         bool ok = true;
         Tile T;
         for (T.set(A, blockIdx.x); T.t < A.tiles && ok; T.set(A, T.t + gridDim.x)) {
             for (int kb = 0; kb < nkb && ok; kb++, it++) {
                 const u32 b = seg & 1, s = it % kStages;
-                if (kb % kbs == 0) ok = mbar_wait(acc_empty + 8 * b, seg >> 1 & 1, &stop);
-                ok = ok && mbar_wait(full + 8 * s, it / kStages & 1, &stop);
+                if (kb % kbs == 0) ok = mbar_wait(acc_empty + 8 * b, seg >> 1 & 1, &stop, A.tries);
+                ok = ok && mbar_wait(full + 8 * s, it / kStages & 1, &stop, A.tries);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -416,15 +416,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
                 if (last) seg++;
             }
         }
-        if (!ok && it > 0 && lane == 0) {   // leaving early: the products under way, bounded
-            int never = 0;
-            mbar_wait(empty + 8 * ((it - 1) % kStages), (it - 1) / kStages & 1, &never);
-        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    // When no wait has run out, the last sums have been read, so every product
+    // is done and every copy has been used.  When one has, a role that had
+    // already finished, or left later, may have copies into this block's shared
+    // memory or products under way: nothing is issued any more, and whoever
+    // issued them waits for them (bounded) before the block can end.
+    if (stop) {
+        if (tid == 17 * 32)   // words: the last use of every slot
+            for (u32 k = it > kRaw ? it - kRaw : 0; k < it; k++) mbar_drain(raw_full + 8 * (k % kRaw), k / kRaw & 1);
+        if (tid == kEpi || tid == kEpi + kGroup) {   // digits: the group's last two slots, unless used again since
+            const u32 grp = tid != kEpi, end = cut_end[grp];
+            for (u32 k = end >= 3 ? end - 3 : end ? end - 1 : 0; k < end; k += 2)
+                if (cut_end[grp ^ 1] < k + kStages + 1) mbar_drain(full + 8 * (k % kStages), k / kStages & 1);
+        }
+        if (tid == 16 * 32 && it > 0) {
+            mbar_drain(empty + 8 * ((it - 1) % kStages), (it - 1) / kStages & 1);
+            if (seg > 0) mbar_drain(acc_full + 8 * ((seg - 1) & 1), (seg - 1) >> 1 & 1);
+        }
+        if (tid == 0) *A.err = 1;
+        __syncthreads();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (stop && tid == 0) *A.err = 1;
     if (warp == 16)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
@@ -587,6 +602,7 @@ void combine(fg_ctx *ctx, const fg_plan *pl, const u64 *X, u64 *Z, int z_ls, int
         A.corr1 = (A.f1 + 63) / 64;
         A.corr_blocks = C.corr_blocks;
         A.accumulate = accumulate || f0 > fb;
+        A.tries = ctx->wait_tries;
         A.tiles = A.nj * (A.N / kTileX) * A.nl * 2;
         for (int i = 0; i < A.nl; i++) A.da[i] = (uint8_t)C.da[i];
         k_comb_mma<<<std::min(A.tiles, sms), kThreads, kSmem, ctx->stream>>>(A);

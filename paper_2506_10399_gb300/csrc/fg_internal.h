@@ -199,6 +199,10 @@ struct fg_ctx {
         int64_t launches = 0;
     } batch;
 
+    // polls after which a kernel's bounded wait gives up; one takes 3.75 us
+    // where nothing arrives (measured), so the default is a second
+    static constexpr uint32_t kWaitTries = 1u << 18;
+    uint32_t wait_tries = kWaitTries;
     // set by a kernel whose bounded wait ran out (page-locked, read by the
     // host after a synchronisation)
     int *wait_err = nullptr;
