@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_comb_mma(const __grid_constant_
                 const u32 s = it % kStages, rs = it % kRaw;
                 ok = mbar_wait(raw_full + 8 * rs, it / kRaw & 1, &stop, A.tries);
                 if (ok && it >= kStages) ok = mbar_wait(empty + 8 * s, (it / kStages - 1) & 1, &stop, A.tries);
+                ok = __all_sync(0xFFFFFFFFu, ok);   // lanes may differ; they meet again below
                 if (!ok) break;
                 if (x == 0) {
                     mbar_arrive_tx(full + 8 * s, bbytes);

@@ -52,3 +52,20 @@ def test_waits_that_give_up_at_once_end_in_a_timeout(F):
         limit(1 << 18)
         assert torch.equal(layer(), want)
     close()
+
+
+@pytest.mark.parametrize("F,Fp", [(96, 16), (300, 48), (1000, 16)])
+@pytest.mark.parametrize("tries", [1, 2, 4, 16])
+def test_waits_that_may_give_up_midway_end_in_a_timeout_or_in_the_words(F, Fp, tries):
+    """A limit of a few polls runs out in some warps and lanes and not in others."""
+    torch, fg, limit, layer, close = setup(F, Fp)
+    want = layer().clone()
+    limit(tries)
+    for _ in range(3):
+        try:
+            assert torch.equal(layer(), want)
+        except fg.FicgcnError as e:
+            assert e.code == ETIMEOUT
+    limit(1 << 18)
+    assert torch.equal(layer(), want)
+    close()
