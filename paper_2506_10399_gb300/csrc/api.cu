@@ -143,6 +143,15 @@ void fg_ctx::check_waits()
     throw fg_error(FG_ETIMEOUT, "a kernel's bounded wait ran out");
 }
 
+void fg_ctx::drop_waits()
+{
+    if (!wait_err) return;
+    cudaStreamSynchronize(stream);
+    for (cudaStream_t st : pool) cudaStreamSynchronize(st);
+    if (batch_stream) cudaStreamSynchronize(batch_stream);
+    *wait_err = 0;
+}
+
 extern "C" int fg_ctx_set_wait_tries(fg_ctx *ctx, uint32_t tries)
 {
     if (!ctx) return FG_EINVAL;

@@ -208,6 +208,7 @@ struct fg_ctx {
     int *wait_err = nullptr;
     int *wait_error();      // its device address
     void check_waits();     // throws FG_ETIMEOUT when it is set, and clears it
+    void drop_waits();      // a call that failed otherwise: its kernels' word must not reach the next call
 
     int L() const { return nq - 1; }
     int ext(int level) const { return level + 1 + np; }

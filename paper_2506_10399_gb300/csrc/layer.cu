@@ -1072,10 +1072,12 @@ static int layer_batch(fg_ctx *ctx, const fg_keys *keys, const fg_plan *const *p
     } catch (const fg_error &e) {
         ctx->stream = home;
         ctx->err = e.what();
+        ctx->drop_waits();
         return e.code;
     } catch (const std::exception &e) {
         ctx->stream = home;
         ctx->err = e.what();
+        ctx->drop_waits();
         return FG_EOOM;
     }
     return FG_OK;
@@ -1113,9 +1115,11 @@ int fg_gcn_layer_axw_seeded(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl,
         if (out_scale) *out_scale = ctx->scale;
     } catch (const fg_error &e) {
         ctx->err = e.what();
+        ctx->drop_waits();
         return e.code;
     } catch (const std::exception &e) {
         ctx->err = e.what();
+        ctx->drop_waits();
         return FG_EOOM;
     }
     return FG_OK;
@@ -1130,9 +1134,11 @@ int fg_gcn_layer_axw(fg_ctx *ctx, const fg_keys *keys, const fg_plan *pl, const 
         if (out_scale) *out_scale = ctx->scale;
     } catch (const fg_error &e) {
         ctx->err = e.what();
+        ctx->drop_waits();
         return e.code;
     } catch (const std::exception &e) {
         ctx->err = e.what();
+        ctx->drop_waits();
         return FG_EOOM;
     }
     return FG_OK;

@@ -2,6 +2,8 @@
 ends, the call returns FG_ETIMEOUT, and the same context then gives the words
 it gave before.  Column counts below, at and above the stages that are under
 way at once, so that a role gives up while another has finished."""
+from types import SimpleNamespace
+
 import numpy as np
 import pytest
 
@@ -9,7 +11,7 @@ from paper_2506_10399_gb300 import workloads as wl
 
 pytestmark = pytest.mark.gpu
 PRM = dict(log_n=10, q_bits=[60, 45, 40, 45], p_bits=[60], alpha=1, log_scale=45)
-ETIMEOUT = -6
+EKEY, ETIMEOUT = -3, -6
 
 
 def setup(F, Fp=16):
@@ -37,35 +39,54 @@ def setup(F, Fp=16):
         for h in (plan, keys, ctx):
             h.close()
 
-    return torch, fg, limit, layer, close
+    return SimpleNamespace(torch=torch, fg=fg, ctx=ctx, keys=keys, plan=plan, x=x, limit=limit, layer=layer, close=close)
 
 
 @pytest.mark.parametrize("F", [40, 96, 97, 300])
 def test_waits_that_give_up_at_once_end_in_a_timeout(F):
-    torch, fg, limit, layer, close = setup(F)
-    want = layer().clone()
+    v = setup(F)
+    want = v.layer().clone()
     for _ in range(2):
-        limit(0)
-        with pytest.raises(fg.FicgcnError) as e:
-            layer()
+        v.limit(0)
+        with pytest.raises(v.fg.FicgcnError) as e:
+            v.layer()
         assert e.value.code == ETIMEOUT
-        limit(1 << 18)
-        assert torch.equal(layer(), want)
-    close()
+        v.limit(1 << 18)
+        assert v.torch.equal(v.layer(), want)
+    v.close()
 
 
 @pytest.mark.parametrize("F,Fp", [(96, 16), (300, 48), (1000, 16)])
 @pytest.mark.parametrize("tries", [1, 2, 4, 16])
 def test_waits_that_may_give_up_midway_end_in_a_timeout_or_in_the_words(F, Fp, tries):
     """A limit of a few polls runs out in some warps and lanes and not in others."""
-    torch, fg, limit, layer, close = setup(F, Fp)
-    want = layer().clone()
-    limit(tries)
+    v = setup(F, Fp)
+    want = v.layer().clone()
+    v.limit(tries)
     for _ in range(3):
         try:
-            assert torch.equal(layer(), want)
-        except fg.FicgcnError as e:
+            assert v.torch.equal(v.layer(), want)
+        except v.fg.FicgcnError as e:
             assert e.code == ETIMEOUT
-    limit(1 << 18)
-    assert torch.equal(layer(), want)
-    close()
+    v.limit(1 << 18)
+    assert v.torch.equal(v.layer(), want)
+    v.close()
+
+
+def test_a_call_that_fails_otherwise_leaves_no_timeout_behind():
+    """A batch whose first query's waits run out and whose second has no
+    rotation key: the call reports the key, and the next call its words."""
+    v = setup(96)
+    want = v.layer().clone()
+    w = wl.make_workload(graph="er", V=16, deg=3.0, F=2, Fp=1, seed=3)
+    rotating = v.fg.plan_build(v.ctx, w.row_ptr, w.col, w.val, w.W, wl.random_order(w.V, v.ctx.slots, 3), t=1)
+    out = v.torch.empty(1, 2, rotating.info()["out_level"] + 1, v.ctx.n, dtype=v.torch.int64, device="cuda")
+    v.limit(0)
+    with pytest.raises(v.fg.FicgcnError) as e:
+        v.fg.gcn_layer_batch(v.ctx, v.keys, [v.plan, rotating], [v.x, v.x[:2].contiguous()],
+                             [v.torch.empty_like(want), out], streams=1, graph=False)
+    assert e.value.code == EKEY
+    v.limit(1 << 18)
+    assert v.torch.equal(v.layer(), want)
+    rotating.close()
+    v.close()
