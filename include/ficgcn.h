@@ -207,6 +207,7 @@ int fg_decrypt_decode(fg_ctx *ctx, const void *sk_blob, size_t sk_len, const uin
 /* Copy the rotation keys of an evk blob to the device (NTT domain) after
  * checking its magic, parameters and checksum (FG_EKEY otherwise). */
 int fg_load_evk(fg_ctx *ctx, const void *evk_blob, size_t len, fg_keys **out);
+/* Keys and plans may be destroyed after their context (not used then). */
 int fg_keys_destroy(fg_keys *keys);
 /* Coefficient-domain copy of key `amount`'s digit j (amount FG_RELIN: the
  * relinearisation key): b and a as [L+1+K][N] (host or device buffers).

@@ -1143,7 +1143,7 @@ int fg_load_evk(fg_ctx *ctx, const void *evk_blob, size_t len, fg_keys **out)
 int fg_keys_destroy(fg_keys *keys)
 {
     if (!keys) return FG_OK;
-    if (keys->ctx) cudaStreamSynchronize(keys->ctx->stream);
+    cudaDeviceSynchronize();   // not the context's stream: the context may be gone
     for (auto &kv : keys->keys) cudaFree(kv.second.d);
     delete keys;
     return FG_OK;

@@ -201,7 +201,7 @@ int fg_plan_build_inter(fg_ctx *ctx, const int32_t *nbr, const double *wts, int 
 int fg_plan_destroy(fg_plan *plan)
 {
     if (!plan) return FG_OK;
-    if (plan->ctx) cudaStreamSynchronize(plan->ctx->stream);
+    cudaDeviceSynchronize();   // not the context's stream: the context may be gone
     for (auto &m : plan->masks) cudaFree(m.d);
     cudaFree(plan->d_comb);
     plan->comb.release();
