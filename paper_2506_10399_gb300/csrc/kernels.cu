@@ -1048,7 +1048,7 @@ static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool
     // finishing: ext read as well, and out when it accumulates
     KTimer kt(ctx, "ntt", (double)active * src.rows * ctx->n * 8 * (fin ? 3 + fin->accumulate : 2));
     if (ctx->log_n < 16) {
-        ntt_small(ctx, bt, count, inverse, fin);
+        ntt_small(ctx, bt, count, active * src.rows, inverse, fin);
         return;
     }
     ntt16_launch(ctx, bt, count, inverse, nullptr, fin);

@@ -388,23 +388,26 @@ void ntt_last_tables(fg_ctx *ctx)
     CUDA_TRY(cudaStreamSynchronize(ctx->stream));
 }
 
-void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin)
+void ntt_small(fg_ctx *ctx, const Batch &bt, int count, int working, bool inverse, const Finish *fin)
 {
     bool one = ctx->log_n <= 11;
     switch (ctx->log_n) {
     case 10: launch_rows<10, 10>(ctx, bt, count, inverse, fin); break;
     case 11: launch_rows<11, 11>(ctx, bt, count, inverse, fin); break;
     case 12:
-        // as at 2^13, below 80 limbs: a rotation (3 to 12 limbs a transform, six
-        // transforms) 118 / 111 us; 96 limbs 12.2 / 13.8 us
-        one = count >= 80;
+        // Whole limbs from 64 limbs to work on (limbs left alone cost a block
+        // that ends at once).  A layer of the toy set, transforms of 8 to 64
+        // limbs, takes 748 us with the line at 16 limbs, 739 at 32 and 720 to
+        // 722 at 48, 64 and 80; a product of eight pairs with 64 of 304 limbs
+        // to work on in its ModDown 245 us in one pass, 260 in two.
+        one = working >= 64;
         if (one) launch_rows<12, 12>(ctx, bt, count, inverse, fin);
         else two_passes<12>(ctx, bt, count, inverse, fin);
         break;
     case 13: {
         // one block a limb leaves most SMs idle below 100 limbs (us: one pass /
         // two, 8 limbs 14.8 / 9.5, 64 14.9 / 12.0, 128 14.6 / 17.6)
-        one = count >= 100;
+        one = working >= 100;
         if (one) launch_rows<13, 13>(ctx, bt, count, inverse, fin);
         else two_passes<13>(ctx, bt, count, inverse, fin);
         break;

@@ -107,5 +107,6 @@ __device__ __forceinline__ void put_pair(u64 w0, u64 w1, u64 *d, size_t pos, con
     *o = r;
 }
 
-// N = 2^10 .. 2^15 (ntt.cu); fin: forward only
-void ntt_small(fg_ctx *ctx, const Batch &bt, int count, bool inverse, const Finish *fin = nullptr);
+// N = 2^10 .. 2^15 (ntt.cu); count limbs, of which `working` are transformed
+// and the others left alone (pidx < 0); fin: forward only
+void ntt_small(fg_ctx *ctx, const Batch &bt, int count, int working, bool inverse, const Finish *fin = nullptr);
