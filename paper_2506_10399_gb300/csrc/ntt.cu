@@ -405,9 +405,15 @@ void ntt_small(fg_ctx *ctx, const Batch &bt, int count, int working, bool invers
         else two_passes<12>(ctx, bt, count, inverse, fin);
         break;
     case 13: {
-        // one block a limb leaves most SMs idle below 100 limbs (us: one pass /
-        // two, 8 limbs 14.8 / 9.5, 64 14.9 / 12.0, 128 14.6 / 17.6)
-        one = working >= 100;
+        // One pass runs one limb an SM at a time, two passes fill the chip at
+        // any count, so one pass pays where its last wave is nearly full (us,
+        // one pass / two, with 6 of event overhead, 45-bit primes forward: 8
+        // limbs 18.8 / 13.8, 104 19.3 / 20.0, 152 19.7 / 22.2, 160 31.0 / 24.0,
+        // 256 30.9 / 31.7, 304 31.0 / 34.5, 312 41.2 / 34.9, 456 43.1 / 44.6,
+        // 480 53.4 / 47.5; inverse and 60-bit primes within 2 us of these).
+        // In whole calls: a product of sixteen pairs, 10 primes, 395 -> 376 us.
+        constexpr int kSms = 152;
+        one = working >= 150 * ((working + kSms - 1) / kSms) - 50;
         if (one) launch_rows<13, 13>(ctx, bt, count, inverse, fin);
         else two_passes<13>(ctx, bt, count, inverse, fin);
         break;
