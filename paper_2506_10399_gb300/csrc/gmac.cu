@@ -371,6 +371,17 @@ k_group_mac_tile(const __grid_constant__ TProg pg, int ncol, int level, int E, i
 
 namespace kern {
 
+// Lets a kernel take more than 48 KB of dynamic shared memory: always up to all
+// a block can have, since the limit belongs to the kernel, and a limit of this
+// launch's own size would undercut a launch that another thread is about to
+// make.  (Not a stream operation: allowed while capturing.)
+template <class K>
+static void allow_shared(K kern, size_t bytes)
+{
+    if (bytes > 48 * 1024)
+        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+}
+
 // more than kGmXs outputs: k_group_mac_tile
 static void group_mac_tile(fg_ctx *ctx, const std::vector<GroupSource> &srcs, const std::vector<Dest> &terms_in,
                            const std::vector<int> &term_dest, const std::vector<u64 *> &outs, bool accumulate, int ncol,
@@ -419,8 +430,7 @@ static void group_mac_tile(fg_ctx *ctx, const std::vector<GroupSource> &srcs, co
     const int v = (ctx->tune.gmac_regs ? 1 : 0) + (ctx->tune.kara ? 2 : 0);
     auto kern = v == 0 ? k_group_mac_tile<2, false> : v == 1 ? k_group_mac_tile<3, false>
               : v == 2 ? k_group_mac_tile<2, true> : k_group_mac_tile<3, true>;
-    if (sm > 48 * 1024)   // a property of the kernel, not a stream operation (allowed while capturing)
-        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_shared(kern, sm);
     kern<<<g, G * kGmacTile, sm, ctx->stream>>>(pg, ncol, level, E, ls, ctx->log_n, ctx->d_primes, ctx->nq);
 }
 
@@ -468,8 +478,7 @@ static void group_mac_stream(fg_ctx *ctx, const std::vector<GroupSource> &srcs, 
     const size_t sm = (size_t)kGmStages * pg.stage_words * 8;
     const dim3 g(npg, N >> pg.lts, E);
     const GmacKernel kern = kGmacKernels[X - 1];
-    if (sm > 48 * 1024)   // a property of the kernel, not a stream operation (allowed while capturing)
-        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_shared(kern, sm);
     kern<<<g, pg.pw << pg.lts, sm, ctx->stream>>>(pg, level, E, ls, ctx->log_n, ctx->d_primes, ctx->nq);
 }
 
