@@ -27,13 +27,11 @@ Batch make_batch(u64 *src, int src_stride, u64 *dst, int dst_stride, int per_row
     return b;
 }
 
-fg_ctx *g_launch_ctx = nullptr;   // context of the wrapper being run (for launch counting)
-
-inline void check_launch(const char *what, int kernels = 1)
+inline void check_launch(fg_ctx *ctx, const char *what, int kernels = 1)
 {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw fg_error(FG_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
-    if (g_launch_ctx) g_launch_ctx->launches += kernels;
+    ctx->launches += kernels;
 }
 
 // ------------------------------------------------------------------------
@@ -964,7 +962,6 @@ namespace kern {
 
 KTimer::KTimer(fg_ctx *c, const char *cls, double alg_bytes) : ctx(c), bytes(alg_bytes)
 {
-    g_launch_ctx = c;
     on = !c->time_class.empty() && c->time_class == cls;
     if (on) {
         a = c->event();
@@ -1052,7 +1049,7 @@ static void launch_ntt(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst, bool
         return;
     }
     ntt16_launch(ctx, bt, count, inverse, nullptr, fin);
-    check_launch("ntt", 2);
+    check_launch(ctx, "ntt", 2);
 }
 
 void ntt_fwd(fg_ctx *ctx, const LimbSet &src, const LimbSet &dst) { launch_ntt(ctx, src, dst, false); }
@@ -1073,7 +1070,7 @@ void to_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx, bo
     k_to_mont<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(contiguous(data, count, pidx),
                                                                ctx->d_primes, ctx->n, split ? 1 : 0,
                                                                times_p ? ctx->d_pmodq : nullptr, ctx->nq);
-    check_launch("to_mont");
+    check_launch(ctx, "to_mont");
 }
 
 void from_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx)
@@ -1082,7 +1079,7 @@ void from_mont(fg_ctx *ctx, u64 *data, int count, const std::vector<int> &pidx)
     KTimer kt(ctx, "from_mont", 0);
     k_from_mont<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(contiguous(data, count, pidx),
                                                                  ctx->d_primes, ctx->n);
-    check_launch("from_mont");
+    check_launch(ctx, "from_mont");
 }
 
 void pointwise(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count,
@@ -1092,7 +1089,7 @@ void pointwise(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count,
     KTimer kt(ctx, "pointwise", 0);
     k_pointwise<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(
         a, b, c, contiguous(c, count, pidx), ctx->d_primes, ctx->n);
-    check_launch("pointwise");
+    check_launch(ctx, "pointwise");
 }
 
 void add(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count, const std::vector<int> &pidx)
@@ -1101,21 +1098,21 @@ void add(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *c, int count, const std::
     KTimer kt(ctx, "add", 0);
     k_add<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(a, b, c, contiguous(c, count, pidx),
                                                            ctx->d_primes, ctx->n);
-    check_launch("add");
+    check_launch(ctx, "add");
 }
 
 void tensor(fg_ctx *ctx, const u64 *a, const u64 *b, u64 *lane, u64 *d1, int n, int nl)
 {
     KTimer kt(ctx, "tensor", (double)n * nl * ctx->n * 8 * (a == b ? 5 : 7));
     k_tensor<<<dim3(ctx->n / 256, nl, n), 256, 0, ctx->stream>>>(a, b, lane, d1, nl, ctx->d_primes, ctx->d_pmodq, ctx->n);
-    check_launch("tensor");
+    check_launch(ctx, "tensor");
 }
 
 void add_part1(fg_ctx *ctx, u64 *u, int E, const u64 *d, int n, int nl)
 {
     KTimer kt(ctx, "add", (double)n * nl * ctx->n * 8 * 3);
     k_add_part1<<<dim3(ctx->n / 256, nl, n), 256, 0, ctx->stream>>>(u, E, d, nl, ctx->d_primes, ctx->n);
-    check_launch("add_part1");
+    check_launch(ctx, "add_part1");
 }
 
 void neg(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &pidx)
@@ -1124,7 +1121,7 @@ void neg(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &p
     KTimer kt(ctx, "neg", 0);
     k_neg<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(a, c, contiguous(c, count, pidx),
                                                            ctx->d_primes, ctx->n);
-    check_launch("neg");
+    check_launch(ctx, "neg");
 }
 
 void scalar(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int> &pidx,
@@ -1134,7 +1131,7 @@ void scalar(fg_ctx *ctx, const u64 *a, u64 *c, int count, const std::vector<int>
     KTimer kt(ctx, "scalar", 0);
     k_scalar<<<ew_grid(ctx->n, count), 256, 0, ctx->stream>>>(
         a, c, contiguous(c, count, pidx), ctx->d_primes, d_scal, ctx->n);
-    check_launch("scalar");
+    check_launch(ctx, "scalar");
 }
 
 void automorphism(fg_ctx *ctx, const u64 *a, u64 *c, int nlimbs, uint32_t g)
@@ -1142,7 +1139,7 @@ void automorphism(fg_ctx *ctx, const u64 *a, u64 *c, int nlimbs, uint32_t g)
     if (!nlimbs) return;
     KTimer kt(ctx, "automorphism", 0);
     k_automorphism<<<ew_grid(ctx->n, nlimbs), 256, 0, ctx->stream>>>(a, c, nlimbs, g, ctx->log_n);
-    check_launch("automorphism");
+    check_launch(ctx, "automorphism");
 }
 
 void small_to_res(fg_ctx *ctx, const int8_t *e, u64 *out, int n_limbs, const int *d_pidx)
@@ -1150,7 +1147,7 @@ void small_to_res(fg_ctx *ctx, const int8_t *e, u64 *out, int n_limbs, const int
     KTimer kt(ctx, "small_to_res", 0);
     k_small_to_res<<<ew_grid(ctx->n, n_limbs), 256, 0, ctx->stream>>>(e, out, d_pidx,
                                                                       ctx->d_primes, ctx->n);
-    check_launch("small_to_res");
+    check_launch(ctx, "small_to_res");
 }
 
 void expand_uniform(fg_ctx *ctx, cudaStream_t st, u64 *ct, size_t ct_pitch, const u64 *c0, int ncols,
@@ -1161,7 +1158,7 @@ void expand_uniform(fg_ctx *ctx, cudaStream_t st, u64 *ct, size_t ct_pitch, cons
     dim3 g((ctx->n + 255) / 256, nl, ncols);
     k_expand_uniform<<<g, 256, 0, st>>>(ct, ct_pitch, c0, nl, seed, hm::kSeededPurpose, index0,
                                         ctx->d_primes, ctx->n);
-    check_launch("expand_uniform");
+    check_launch(ctx, "expand_uniform");
 }
 
 void copy_limbs(fg_ctx *ctx, const u64 *src, int src_ls, u64 *dst, int dst_ls, int npoly, int nl)
@@ -1170,7 +1167,7 @@ void copy_limbs(fg_ctx *ctx, const u64 *src, int src_ls, u64 *dst, int dst_ls, i
     KTimer kt(ctx, "copy", (double)npoly * nl * ctx->n * 16);
     dim3 g((ctx->n + 255) / 256, nl, npoly);
     k_copy_limbs<<<g, 256, 0, ctx->stream>>>(src, src_ls, dst, dst_ls, nl, ctx->n);
-    check_launch("copy_limbs");
+    check_launch(ctx, "copy_limbs");
 }
 
 void comb_const_mac(fg_ctx *ctx, const u64 *X, int F, int Fp, int level, const u64 *consts, u64 *Z,
@@ -1186,7 +1183,7 @@ void comb_const_mac(fg_ctx *ctx, const u64 *X, int F, int Fp, int level, const u
     dim3 g(((ctx->n + 255) / 256) * nj, level + 1, 2);
     k_comb<<<g, 256, 0, ctx->stream>>>(X, F, fb, fe, accumulate ? 1 : 0, Fp, nj, level, consts, Z, z_ls,
                                        ctx->d_primes, ctx->n);
-    check_launch("comb");
+    check_launch(ctx, "comb");
 }
 
 void rescale_coef(fg_ctx *ctx, const u64 *in, int in_ls, u64 *out, int out_ls, int npoly, int level)
@@ -1196,7 +1193,7 @@ void rescale_coef(fg_ctx *ctx, const u64 *in, int in_ls, u64 *out, int out_ls, i
     dim3 g((ctx->n + 255) / 256, level, npoly);
     k_rescale_coef<<<g, 256, 0, ctx->stream>>>(in, in_ls, out, out_ls, level, ctx->d_primes,
                                                ctx->rescale_tab(level), ctx->n);
-    check_launch("rescale_coef");
+    check_launch(ctx, "rescale_coef");
 }
 
 void rescale_ntt(fg_ctx *ctx, u64 *ct, int ls, int npoly, int level)
@@ -1213,7 +1210,7 @@ void rescale_ntt(fg_ctx *ctx, u64 *ct, int ls, int npoly, int level)
     {
         KTimer kt(ctx, "rescale", (double)npoly * (level + 1) * N * 8);
         k_bcast_reduce<<<g, 256, 0, ctx->stream>>>(ct, ls, level, rr, level, ctx->d_primes, N);
-        check_launch("bcast_reduce");
+        check_launch(ctx, "bcast_reduce");
     }
     std::vector<int> pid(level);
     for (int i = 0; i < level; i++) pid[i] = i;
@@ -1222,7 +1219,7 @@ void rescale_ntt(fg_ctx *ctx, u64 *ct, int ls, int npoly, int level)
     KTimer kt(ctx, "rescale", (double)npoly * level * N * 8 * 3);
     k_rescale_finish<<<g, 256, 0, ctx->stream>>>(ct, ls, rr, level, ctx->d_primes,
                                                  ctx->rescale_tab(level), N);
-    check_launch("rescale_finish");
+    check_launch(ctx, "rescale_finish");
 }
 
 // ModUp at N = 2^16 with the conversion fused into the digits' first NTT
@@ -1240,7 +1237,7 @@ static void modup16_fused(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int le
         Batch bt = make_batch(const_cast<u64 *>(lane) + (size_t)ls * N, 2 * ls, y, nl, nl, ncol, pid);
         KTimer kt(ctx, "ntt", (double)nl * ncol * N * 8 * 2);
         ntt16_launch(ctx, bt, ncol * nl, true, ctx->modup_scale_tab(level));
-        check_launch("ntt", 2);
+        check_launch(ctx, "ntt", 2);
     }
     const int nmax = std::min(ctx->alpha, nl);
     int n_out = 0;
@@ -1260,7 +1257,7 @@ static void modup16_fused(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int le
                                                                    ctx->d_primes, fwd)
         FG_NIN_DISPATCH(nmax, FG_LAUNCH)
 #undef FG_LAUNCH
-        check_launch("modup_ntt16_a");
+        check_launch(ctx, "modup_ntt16_a");
     }
     std::vector<int> dp(beta * E);
     for (int d = 0; d < beta; d++)
@@ -1271,7 +1268,7 @@ static void modup16_fused(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int le
     for (int v : dp) active += v >= 0;
     KTimer kt(ctx, "ntt", (double)active * ncol * N * 8 * 2 / 2);
     ntt16_pass_b_od<OD>(ctx, bd, ncol * beta * E);
-    check_launch("ntt16_fwd_b");
+    check_launch(ctx, "ntt16_fwd_b");
 }
 
 void modup(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level, u64 *digits)
@@ -1296,7 +1293,7 @@ void modup(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level, u64 *digit
                                                 ctx->d_primes, N)
     FG_NIN_DISPATCH(std::min(ctx->alpha, nl), FG_LAUNCH)
 #undef FG_LAUNCH
-    check_launch("modup_conv");
+    check_launch(ctx, "modup_conv");
     }
     std::vector<int> dp(beta * E);
     for (int d = 0; d < beta; d++)
@@ -1325,7 +1322,7 @@ void rotate(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, i
                                                    ctx->d_primes, N)
     FG_NIN_DISPATCH(ctx->np, FG_LAUNCH)
 #undef FG_LAUNCH
-    check_launch("moddown_conv");
+    check_launch(ctx, "moddown_conv");
     }
     std::vector<int> pq(nl);
     for (int i = 0; i < nl; i++) pq[i] = i;
@@ -1335,7 +1332,7 @@ void rotate(fg_ctx *ctx, const KeyDev &key, const u64 *lane, int ls, int ncol, i
     KTimer kt(ctx, "moddown_mac", (double)7 * ncol * nl * N * 8);
     k_moddown_finish<<<g3, 256, 0, ctx->stream>>>(u, E, conv, lane, ls, ncol, level, key.galois, ctx->log_n,
                                                   ctx->pinv_tab(level), out, out_ls, ctx->d_primes);
-    check_launch("moddown_finish");
+    check_launch(ctx, "moddown_finish");
 }
 
 void stay_mac(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level,
@@ -1355,7 +1352,7 @@ void stay_mac(fg_ctx *ctx, const u64 *lane, int ls, int ncol, int level,
         KTimer kt(ctx, "stay_mac", ((double)2 * ncol * nl + (double)dl.n * nl +
                                      (double)dl.n * ncol * 2 * nl * 2) * N * 8);
         k_stay_mac<<<g, 256, 0, ctx->stream>>>(lane, ls, ncol, level, dl, ctx->d_primes, N);
-        check_launch("stay_mac");
+        check_launch(ctx, "stay_mac");
     }
 }
 
@@ -1366,7 +1363,7 @@ void lift_special(fg_ctx *ctx, const u64 *limb0, u64 *out)
     k_lift_special<<<ew_grid(ctx->n, ctx->np), 256, 0, ctx->stream>>>(limb0, ctx->primes[0], out,
                                                                       ctx->np, ctx->nq,
                                                                       ctx->d_primes, ctx->n);
-    check_launch("lift_special");
+    check_launch(ctx, "lift_special");
 }
 
 // ModDown + rescale at N = 2^16 with the conversion fused into w's first
@@ -1382,7 +1379,7 @@ static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out
         Batch bt = make_batch(ext, E, ext, E, E, npoly, pp);
         KTimer kt(ctx, "ntt", (double)npoly * (ctx->np + 1) * N * 8 * 2);
         ntt16_launch(ctx, bt, npoly * E, true, ctx->moddown_scale_tab(level));
-        check_launch("ntt", 2);
+        check_launch(ctx, "ntt", 2);
     }
     u64 *w = (u64 *)ctx->buf("ks_conv", (size_t)npoly * l * N * 8);
     const ConvTab *tab = ctx->moddown_tab(level);
@@ -1394,7 +1391,7 @@ static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out
         k_moddown_prep<M><<<g1, 256, 0, ctx->stream>>>(ext, E, l, tab, ctx->pinv_tab(level), hq, ctx->d_primes, N)
         FG_NIN_DISPATCH(ctx->np, FG_LAUNCH)
 #undef FG_LAUNCH
-        check_launch("moddown_prep");
+        check_launch(ctx, "moddown_prep");
         dim3 g2(16, l, npoly);
 #define FG_LAUNCH(M)                                                                                \
         k_moddown_ntt16_a<M, OD><<<g2, 256, 0, ctx->stream>>>(ext, E, w, l, tab, ctx->d_pmodq, hq,    \
@@ -1402,7 +1399,7 @@ static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out
                                                               (const ulonglong2 *)ctx->d_fwd)
         FG_NIN_DISPATCH(ctx->np, FG_LAUNCH)
 #undef FG_LAUNCH
-        check_launch("moddown_ntt16_a");
+        check_launch(ctx, "moddown_ntt16_a");
     }
     {
         std::vector<int> pq(l);
@@ -1411,7 +1408,7 @@ static void moddown16_fused(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *out
         const Finish fin{ext, out, ctx->moddown_rescale_tab(level), E, ls, accumulate ? 1 : 0};
         KTimer kt(ctx, "ntt", (double)npoly * l * N * 8 * (2 + fin.accumulate));
         ntt16_pass_b_od<OD>(ctx, bw, npoly * l, &fin);
-        check_launch("ntt16_fwd_b");
+        check_launch(ctx, "ntt16_fwd_b");
     }
 }
 
@@ -1440,7 +1437,7 @@ void moddown_rescale_to_lane(fg_ctx *ctx, u64 *ext, int ncol, int level, u64 *ou
                                                                ctx->d_primes, N)
         FG_NIN_DISPATCH(ctx->np, FG_LAUNCH)
 #undef FG_LAUNCH
-        check_launch("moddown_rescale_conv");
+        check_launch(ctx, "moddown_rescale_conv");
     }
     std::vector<int> pq(l);
     for (int i = 0; i < l; i++) pq[i] = i;

@@ -28,16 +28,21 @@ def test_layers_of_two_threads(V, radix, widths):
         keys = fg.load_evk(ctx, fg.keygen(ctx, 1, plan.rotation_amounts())[1])
         x = torch.stack([torch.randint(0, q, (2, 2, ctx.n), device="cuda") for q in ctx.q], 2).contiguous()
         torch.cuda.synchronize()
+        n0 = ctx.launch_count()
         want = fg.gcn_layer_axw(ctx, keys, plan, x)[0].clone()
+        launches = ctx.launch_count() - n0
         torch.cuda.synchronize()
-        work.append((ctx, keys, plan, x, want, stream))
+        work.append((ctx, keys, plan, x, want, stream, launches))
     failures = []
 
-    def loop(ctx, keys, plan, x, want, stream):
+    def loop(ctx, keys, plan, x, want, stream, launches):
         out = torch.empty_like(want)
         try:
+            n0 = ctx.launch_count()
             for _ in range(2000):
                 fg.gcn_layer_axw(ctx, keys, plan, x, out=out)
+            if ctx.launch_count() - n0 != 2000 * launches:
+                failures.append("launches counted on another context")
             with torch.cuda.stream(stream):
                 if not torch.equal(out, want):
                     failures.append("words differ")
