@@ -29,6 +29,18 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// an output that a kernel may write: memory of the context's own GPU (another
+// GPU's is copied to, which needs no peer mapping)
+bool is_own_ptr(const fg_ctx *ctx, const void *p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == ctx->device);
+}
+
 // a device view of a caller buffer: the buffer itself, or a staged copy
 const u64 *stage_in(fg_ctx *ctx, const u64 *p, size_t words, const char *name)
 {
@@ -1188,7 +1200,7 @@ int fg_poly_mul(fg_ctx *ctx, const uint64_t *a, const uint64_t *b, int level, ui
     kern::ntt_fwd(ctx, sa, ta_s);
     kern::ntt_fwd(ctx, sb, tb_s);
     kern::pointwise(ctx, ta, tb, ta, nl, pid);
-    u64 *o = is_device_ptr(c) ? c : ta;   // the operands have been read
+    u64 *o = is_own_ptr(ctx, c) ? c : ta;   // the operands have been read
     kern::LimbSet os{o, nl, nl, 1, pid};
     kern::ntt_inv(ctx, ta_s, os);
     stage_out(ctx, c, o, (size_t)nl * N);
@@ -1311,7 +1323,7 @@ int fg_rotate(fg_ctx *ctx, const fg_keys *keys, const uint64_t *ct, int level, i
                                   (size_t)ctx->n_digits(level) * ctx->ext(level) * N * 8);
     kern::modup(ctx, lane, nl, 1, level, digits);
     kern::rotate(ctx, key, lane, nl, 1, level, digits, res, nl);
-    u64 *o = is_device_ptr(out) ? out : res;   // the input has been read
+    u64 *o = is_own_ptr(ctx, out) ? out : res;   // the input has been read
     kern::LimbSet rs{res, nl, nl, 2, pid}, os{o, nl, nl, 2, pid};
     kern::ntt_inv(ctx, rs, os);
     stage_out(ctx, out, o, (size_t)2 * nl * N);
