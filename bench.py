@@ -361,16 +361,18 @@ def alu_roofline(fg, ctx, plan, breakdown, F, Fp, alpha, kara=1):
     (fg_int_mul_peak, eight independent chains per thread on every SM), the
     faster of mad.wide.u32 and the carry-chained mad.lo.cc.u32 / madc.hi.u32
     pair; the pair's rate is reported beside it.
-    Achieved: the 32 x 32-bit products of the sums, counted on the plan, over
-    the kernel class's measured time in one layer.  A product of two split
-    words counts four 32 x 32-bit products (lo x lo, lo x hi, hi x lo, hi x
-    hi), three in the group MAC's Karatsuba form (limbs below 2^46, when kara
-    is set); the key switch takes three there too and is still counted with
-    four, and the combination runs on the tensor cores where its shape
-    allows (main leaves it out of the line then):
+    "performed": the 32 x 32-bit products that the kernel's sums take, counted
+    on the plan; "achieved": these over the kernel class's measured time in
+    one layer.  A product of two split words takes four 32 x 32-bit products
+    (lo x lo, lo x hi, hi x lo, hi x hi), three in Karatsuba's form (limbs
+    below 2^46; in the group MAC when kara is set, in the key switch always).
+    "mults" counts the key switch with four everywhere.  The combination runs
+    on the tensor cores where its shape allows (comb_on_tensor_cores; main
+    leaves it out of the line then):
       group_mac: terms x 2F' polynomials x N x (3 or 4 per limb of the E
                  extended limbs at the group's level);
-      ks_ip:     rotations x F' columns x E limbs x N x 2 parts x beta digits x 4;
+      ks_ip:     rotations x F' columns x N x 2 parts x beta digits x (3 or 4
+                 per limb of E);
       comb:      F x F' x 2 parts x (L+1) limbs x N x 4 (the 60-bit limb's
                  64 x 64-bit products counted as four as well).
     Instruction counts of the integer pipes from ncu, where captured, are in
@@ -385,6 +387,7 @@ def alu_roofline(fg, ctx, plan, breakdown, F, Fp, alpha, kara=1):
     N, np_ = ctx.n, ctx.np
     small = [q < (1 << 46) for q in ctx.q]
     prods = {"group_mac": 0.0, "ks_ip": 0.0, "comb": 4.0 * F * Fp * 2 * (int(rec[7]) + 1) * N}
+    ks_done = 0.0
     for _ in range(int(rec[11])):
         lvl, nrot = int(rec[i + 2]), int(rec[i + 5])
         E = lvl + 1 + np_
@@ -395,15 +398,24 @@ def alu_roofline(fg, ctx, plan, breakdown, F, Fp, alpha, kara=1):
         per_limb = sum((3 if (kara and small[j]) else 4) for j in range(lvl + 1)) + 4 * np_
         prods["group_mac"] += float(nterm) * 2 * Fp * N * per_limb
         prods["ks_ip"] += 4.0 * nrot * Fp * E * N * 2 * beta
+        ks_done += float(nrot) * Fp * N * 2 * beta * (sum(3 if small[j] else 4 for j in range(lvl + 1)) + 4 * np_)
     out = {"unit": "32x32-bit multiply-accumulates/s", "peak": peak,
            "peak_kind": "measured (fg_int_mul_peak, the faster of mad.wide.u32 and the carry-chained pair)", "peak_carry_chained_pair": pair,
            "kernels": {}}
     for k, pr in prods.items():
         ms = breakdown.get(k, {}).get("ms") or 0
         if ms > 0:
-            a = pr / (ms / 1e3)
-            out["kernels"][k] = {"achieved": a, "frac": round(a / peak, 4), "mults": pr}
+            done = ks_done if k == "ks_ip" else pr
+            a = done / (ms / 1e3)
+            out["kernels"][k] = {"achieved": a, "frac": round(a / peak, 4), "performed": done, "mults": pr}
     return out
+
+
+def comb_on_tensor_cores(F, Fp, t):
+    """Whether the combination of a layer on device inputs takes the tensor
+    cores: unpacked columns (t = 1), and columns x blocks of 8 outputs at
+    least 40 x blocks of 16 outputs."""
+    return t == 1 and F * -(-Fp // 8) >= 40 * -(-Fp // 16)
 
 
 # ------------------------------------------------------------------ GPU arm
@@ -500,7 +512,8 @@ def run_ours(args):
     dominant = max(breakdown, key=lambda k: breakdown[k]["ms"])
     alu = alu_roofline(fg, ctx, plan, breakdown, w.X.shape[1], Fp=info["n_out"], alpha=c["alpha"],
                        kara=fg.batch_tuning(ctx)[0]["kara"])
-    alu["kernels"].pop("comb", None)   # this shape's combination runs on the tensor cores
+    if comb_on_tensor_cores(w.X.shape[1], info["n_out"], info["t"]):
+        alu["kernels"].pop("comb", None)   # not integer products
 
     # ---- timed region: K steps, HBM-resident inputs
     clocks = Clocks(local)
