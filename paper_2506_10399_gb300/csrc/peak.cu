@@ -29,8 +29,9 @@ __global__ void __launch_bounds__(256) k_mul_peak(u64 *out, u32 seed)
     }
     for (int it = 0; it < kPeakIters; it++) {
         // a new factor, or the product of two loop constants is computed once and the
-        // loop measures 64-bit additions (1.94e13 per second instead of 8.2e12)
-        if (OP == 0) b ^= (u32)it;
+        // loop measures 64-bit additions (1.94e13 per second instead of 8.2e12);
+        // OP 1 feeds its results back
+        if (OP != 1) b ^= (u32)it;
 #pragma unroll
         for (int c = 0; c < kPeakChains; c++) {
             if (OP == 0) {   // 32 x 32 -> 64-bit multiply-add (the split products' step)
