@@ -101,7 +101,7 @@ void fg_free(void *blob);
 /* Instrumentation (no counterpart in the paper, which times on one CPU
  * thread).  fg_ctx_time_kernels: from now on record a CUDA event pair on the
  * context's stream around every call of one kernel class -- "ntt" (one call
- * = the two kernels of a batched transform), "ks_ip", "moddown_conv",
+ * = the one or two kernels of a batched transform), "ks_ip", "moddown_conv",
  * "moddown_mac", "modup_conv", "comb", "rescale", "stay_mac" -- with the
  * call's algorithmic bytes (each operand read once, each result written
  * once); NULL or "" stops.  Earlier records are dropped.

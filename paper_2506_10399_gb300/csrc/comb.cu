@@ -29,13 +29,12 @@
 // of 256 TMEM columns let a segment's products run while the previous one is
 // read.
 //
-// Measured on 500 columns, 16 outputs, 6 limbs, N = 2^16: 0.96 ms, 3.4 TB/s of
-// X (k_comb: 4.0 ms).  Neither HBM nor the tensor cores (19% busy) are full: a
-// stage of 16 KB takes 1500 cycles where its copies alone take 660 and the
-// cutting or the products alone, with the copies, about 1200.  A plain copy
-// needs 128 KB in flight per SM to reach 6.5 TB/s at this stride; six stages
-// hold 96 KB.  Copies of 1 KB rows instead of boxes, words through registers
-// or cp.async instead of TMA, other splits of the ring: all slower by 3 to 30%.
+// Measured on 500 columns, 16 outputs, 6 limbs, N = 2^16: 0.90 ms, 3.5 TB/s of
+// X (k_comb: 4.2 ms).  Neither HBM nor the tensor cores (19% busy) are full: a
+// stage of 16 KB takes 1450 cycles, its copies alone 820 (6.2 TB/s), copies and
+// cutting 1110, copies and products 1310.  Copies of 1 KB rows instead of
+// boxes, words through registers or cp.async instead of TMA, other splits of
+// the ring: all slower by 3 to 30%.
 #include <algorithm>
 #include <cstring>
 

@@ -145,7 +145,8 @@ __device__ __forceinline__ u64 mad_wide(u32 x, u32 y, u64 a)
 // against 60 with it, and nine products either way).  The total S of T < 2^16
 // products of reduced factors is below T q^2, so S / 2^64 < T q (q / 2^64) < q
 // / 4 for q < 2^46, and the result, S / 2^64 plus less than q, needs one
-// subtraction.  The sums stay below 2^62 + 2^46 + 2^41.
+// subtraction.  A0 and A2 stay below 2^62 plus the steps' carries, A1, two
+// products below 2^46 a term, below 2^63 + 2^47.
 __device__ __forceinline__ u64 fold_split(u64 a0, u64 a1, u64 a2, const PrimeC &P)
 {
     const u32 q0 = (u32)P.q & 0x7FFFFF, q1 = (u32)(P.q >> 23), n = (u32)P.qneg;

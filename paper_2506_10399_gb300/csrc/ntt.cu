@@ -6,7 +6,8 @@
 // exchanges (radix-16 rounds, or two radix-8 groups).
 //   * Up to N = 2^13 one block transforms a whole limb: one launch and one
 //     read and write of global memory per transform.
-//   * N = 2^14, 2^15 and small batches at 2^12 and 2^13 take two passes: the first
+//   * N = 2^14, 2^15, small batches at 2^12 and 2^13 and batches at 2^13 whose
+//     last wave of whole limbs would be far from full take two passes: the first
 //     seven stages on 128-row columns (16 columns a block), the rest inside rows
 //     of 32 to 256 (2048 elements a block).
 // The last round's twiddles, one set per thread, come from a table of their own
