@@ -396,12 +396,14 @@ void ntt_small(fg_ctx *ctx, const Batch &bt, int count, int working, bool invers
     case 10: launch_rows<10, 10>(ctx, bt, count, inverse, fin); break;
     case 11: launch_rows<11, 11>(ctx, bt, count, inverse, fin); break;
     case 12:
-        // Whole limbs from 64 limbs to work on (limbs left alone cost a block
-        // that ends at once).  A layer of the toy set, transforms of 8 to 64
-        // limbs, takes 748 us with the line at 16 limbs, 739 at 32 and 720 to
-        // 722 at 48, 64 and 80; a product of eight pairs with 64 of 304 limbs
-        // to work on in its ModDown 245 us in one pass, 260 in two.
-        one = working >= 64;
+        // Two passes below 80 limbs: a rotation (3 to 12 limbs a transform, six
+        // transforms) 118 / 111 us; 96 limbs 12.2 / 13.8 us.  Limbs left alone
+        // count here: in two passes they cost four blocks instead of one, and
+        // with the line at 80 or 64 working limbs a product of eight pairs (64
+        // of 304 limbs at work in its ModDown) took 255 instead of 248 us, or a
+        // batch of three small queries (72 limbs, all at work) 4.07 instead of
+        // 4.03 ms.
+        one = count >= 80;
         if (one) launch_rows<12, 12>(ctx, bt, count, inverse, fin);
         else two_passes<12>(ctx, bt, count, inverse, fin);
         break;

@@ -1,6 +1,6 @@
-"""How many passes a transform at N = 2^12 or 2^13 takes: by the limbs it works
-on, not by those it leaves alone, and by how full the last wave of one limb an
-SM is.  A product of eight pairs (12 limbs a polynomial, of
+"""How many passes a transform at N = 2^12 or 2^13 takes: at 2^13 by the limbs
+it works on, not by those it leaves alone, and by how full the last wave of one
+limb an SM is.  A product of eight pairs (12 limbs a polynomial, of
 which ModDown transforms four) by its launches, and word for word the products
 one at a time, whose transforms take the other form."""
 import pytest
@@ -11,7 +11,7 @@ NQ, NP, ALPHA, PAIRS = 9, 3, 3, 8
 
 def passes(log_n, limbs):
     if log_n == 12:
-        return 1 if limbs >= 64 else 2
+        return 1 if limbs >= 80 else 2
     waves = -(-limbs // 152)
     return 1 if limbs >= 150 * waves - 50 else 2
 
@@ -48,7 +48,7 @@ def test_limbs_left_alone_do_not_count():
     ctx.close()
 
 
-@pytest.mark.parametrize("log_n,limbs", [(12, 63), (12, 64), (13, 99), (13, 100), (13, 152), (13, 153), (13, 249),
+@pytest.mark.parametrize("log_n,limbs", [(12, 79), (12, 80), (13, 99), (13, 100), (13, 152), (13, 153), (13, 249),
                                          (13, 250), (13, 305), (13, 400)])
 def test_both_sides_of_every_line(log_n, limbs):
     """The batch's words against each limb's own transform (two passes)."""
